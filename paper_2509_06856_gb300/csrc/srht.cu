@@ -19,9 +19,10 @@
 // (64 KB).  Each CTA applies the butterflies of the low LOGM row bits in registers
 // (two register stages with one shared-memory exchange); the top LOGQ bits are
 // combined across the cluster through distributed shared memory.  Global loads and
-// stores move whole row segments (C = 32 FP32 or 16 FP64 columns = 128 bytes) so
-// every warp access is coalesced.  The work is adds/subtracts only: HBM-bound in
-// FP32, FP64-ALU-bound in FP64 on this part.
+// stores move whole row segments (C = 32 FP32 columns = 128 bytes) so every warp access
+// is coalesced.  The work is adds/subtracts only: HBM-bound in FP32, FP64-ALU-bound in
+// FP64 on this part, so FP64 groups of 2^8 rows and more run in fixed point on the integer
+// pipe (srht64.cu).
 //
 // Cluster synchronisation: a tile is published through an mbarrier per CTA (one thread
 // fences at cluster scope after a CTA barrier and signals every peer; all threads wait with
@@ -33,7 +34,7 @@
 
 #include <type_traits>
 
-#include "slse_internal.cuh"
+#include "srht_args.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -43,32 +44,6 @@ namespace {
 // Output tag for the FP8 form of the sketch: E4M3 values with one power-of-two scale per
 // 32-column block of a row (scale byte = exponent + 127); the rows' Y values stay BF16.
 struct mx8 {};
-
-struct GroupArgs {
-  const void *in;       // X (pass 1 / single) or W (pass 2)
-  int64_t ldin;
-  const void *in_y;     // Y or WY
-  int64_t N;            // gather mode: rows >= N are the zero padding
-  const int32_t *Psd;   // non-null: gather mode (sign-folded permutation)
-  int64_t istride, igstride;  // input row j = rho * istride + g * igstride
-  void *out;
-  int64_t ldout;
-  void *out_y;
-  const int32_t *pos;   // non-null: output row = pos[k], skipped when < 0
-  int64_t ostride, ogstride;  // output index k = kappa * ostride + g * ogstride
-  int d;
-  int nslab;
-  int logq;
-  int vec_in, vec_out;  // 1: rows allow VEC-wide vector access
-  uint8_t *out_scale;   // FP8 form: block exponents, ld_scale bytes per row
-  int64_t ld_scale;
-  __nv_bfloat16 *hat_out;  // FP8 form: output rows >= hat_row0 go here in BF16 (nullable)
-  int64_t hat_row0, hat_ld;
-  double scale;
-  void *copy_out;       // pass 1 reading host memory: every input row segment is also stored
-                        // here at the same element offset (the device copy of X)
-  unsigned *status;     // nullable: ST_TIMEOUT is raised here when a bounded wait gave up
-};
 
 // Smallest k with amax <= 448 2^k (448 = 1.75 2^8, the largest E4M3 value), clamped to
 // the E8M0 range; -127 for amax = 0.  Exact, from the float's bit fields.
@@ -299,33 +274,12 @@ __global__ void __launch_bounds__(NT, MINB) k_group(const GroupArgs a) {
     const int col = col0 + cq * VA;
     Ts v[VA][RA];
     if (fast_in) {
-      if constexpr (sizeof(Tin) == 4 && sizeof(Ts) == 8 && Q > 1 && !CPY) {
-        // FP64 arithmetic on FP32 storage (clustered sizes, device input): widened on the
-        // integer pipe (the FP64 pipe bounds this pass), the rare denormal, infinity or NaN
-        // with the conversion instruction
-        bool special = false;
 #pragma unroll
-        for (int k = 0; k < RA; ++k) {
-          const Tin *p = in + s_off[b + (k << S1)] + col;
+      for (int k = 0; k < RA; ++k) {
+        Ts t[VA];
+        load_vec<Tin, Ts, VA>(in + s_off[b + (k << S1)] + col, t);
 #pragma unroll
-          for (int e = 0; e < VA; ++e) v[e][k] = widen(__ldcs(p + e), special);
-        }
-        if (__any_sync(__activemask(), special)) {
-#pragma unroll
-          for (int k = 0; k < RA; ++k) {
-            const Tin *p = in + s_off[b + (k << S1)] + col;
-#pragma unroll
-            for (int e = 0; e < VA; ++e) v[e][k] = (Ts)p[e];
-          }
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < RA; ++k) {
-          Ts t[VA];
-          load_vec<Tin, Ts, VA>(in + s_off[b + (k << S1)] + col, t);
-#pragma unroll
-          for (int e = 0; e < VA; ++e) v[e][k] = t[e];
-        }
+        for (int e = 0; e < VA; ++e) v[e][k] = t[e];
       }
       if constexpr (CPY) {
 #pragma unroll
@@ -642,7 +596,16 @@ template <class Tin, class Ts, class Tout, int VA, int VB, int VO, int SLAB_BYTE
 cudaError_t launch_pass_t(const GroupArgs &a, int L, int64_t ngroups, cudaStream_t s) {
   constexpr int CP = SLAB_BYTES / (int)sizeof(Ts);
   cudaError_t e;
-  switch (L) {
+  if constexpr (sizeof(Ts) == 8) {
+    // FP64: from 2^8 rows a group on the integer pipe (srht64.cu: 2^10 rows, d = 200, 4.4 -> 1.7 ms
+    // a pass); smaller groups (N' <= 2^15) do not fill its warps and take tens of microseconds
+    switch (L) {
+      case 5: e = launch_group_t<Tin, Ts, Tout, 5, 1, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s); break;
+      case 6: e = launch_group_t<Tin, Ts, Tout, 6, 1, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s); break;
+      case 7: e = launch_group_t<Tin, Ts, Tout, 7, 1, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s); break;
+      default: e = launch_group_fix<Tin>(a, L, ngroups, s);
+    }
+  } else switch (L) {
     case 5: e = launch_group_t<Tin, Ts, Tout, 5, 1, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s); break;
     case 6: e = launch_group_t<Tin, Ts, Tout, 6, 1, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s); break;
     case 7: e = launch_group_t<Tin, Ts, Tout, 7, 1, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s); break;
