@@ -67,24 +67,6 @@ template <> struct Vec<float, 1> {
     o[0] = stream ? __ldcs(p) : __ldg(p);
   }
 };
-template <> struct Vec<double, 2> {
-  static __device__ __forceinline__ void load(const double *p, double (&o)[2], bool stream) {
-    const double2 t = stream ? __ldcs(reinterpret_cast<const double2 *>(p)) : __ldg(reinterpret_cast<const double2 *>(p));
-    o[0] = t.x; o[1] = t.y;
-  }
-};
-template <> struct Vec<double, 1> {
-  static __device__ __forceinline__ void load(const double *p, double (&o)[1], bool stream) {
-    o[0] = stream ? __ldcs(p) : __ldg(p);
-  }
-};
-template <> struct Vec<float, 2> {  // FP32 data widened to FP64 arithmetic uses float pairs
-  static __device__ __forceinline__ void load(const float *p, float (&o)[2], bool stream) {
-    const float2 t = stream ? __ldcs(reinterpret_cast<const float2 *>(p)) : __ldg(reinterpret_cast<const float2 *>(p));
-    o[0] = t.x; o[1] = t.y;
-  }
-};
-
 template <class T> __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
@@ -138,14 +120,107 @@ __device__ __forceinline__ void warp_sum_rows(double (&v)[R], int lane) {
   for (int q = 0; q < R; ++q) v[q] = tot[q];
 }
 
-// FP32 storage is widened by `widen` (integer pipe): the conversion instruction cost this pass
-// more than its two FP64 FMAs per element (at 2^21 x 512: 6.8 ms from FP32 storage against
-// 4.1 ms from FP64 storage, before the change).
+// The FP64 pipe (two fused multiply-adds per clock and SM on this part) bounds this pass: x_i beta
+// and x_i r_i are one each per element.  So x_i beta is formed on the integer pipes instead, beside
+// the FP64 pipe, which is left with x_i r_i and a handful of operations per row group:
+//  - beta_j = (bh 2^26 + bl) 2^(be - 1075), signed 27- and 26-bit parts, once per pass;
+//  - the row's terms are aligned to the largest exponent F of x_ij beta_j over the row: x_ij's
+//    mantissa becomes the 62-bit integer (zh 2^31 + zl) 2^(F - be ..), bits below 2^-61 of the
+//    row's largest term are dropped;
+//  - zh bh, zh bl and zl bh are summed exactly in 64 bits (three 32 x 32 + 64 bit multiply-adds;
+//    zl bl, at most 2^-58 of the largest term, is left out), the lanes' 96-bit sums are added
+//    exactly in 26-bit pieces, and the total is rounded to FP64 once.
+// The error of x_i beta is then below that of an FP64 chain (2^-53 of the partial sums at each of
+// its d steps): sqrt(d) 2^-60 of the row's largest term, and half an ulp.  A row group with a
+// denormal, an infinity or a NaN, or whose largest product is outside [2^-846, 2^954], takes the FP64
+// sums (warp-uniform).
+// Measured (GB300): N = 2^20, d = 256 FP64 1.07 -> 0.63 ms, d = 512 FP64 2.00 -> 1.17 ms, FP32 storage
+// 2.03 -> 1.23 ms; N = 700001, d = 200 0.725 -> 0.436 ms.  What bounds it now: the FP64 pipe, 0.76
+// busy (the integer pipe 0.67).  Without the ring (rows prefetched into registers) 0.69 ms at 2^20 x
+// 256, without any prefetch 0.86 ms, with three CTAs of 80 registers 0.77 ms.
+struct BetaFix {
+  int bh, bl, be;
+};
+
+constexpr int kNoTerm = -(1 << 20);  // exponent of a zero term
+
+__device__ __forceinline__ BetaFix beta_fix(double b) {
+  const uint32_t hi = (uint32_t)__double2hiint(b), lo = (uint32_t)__double2loint(b);
+  const int e = (int)((hi >> 20) & 0x7FFu);
+  if (e == 0 || e == 0x7FF) return BetaFix{0, 0, e == 0 && ((hi << 1) | lo) == 0u ? kNoTerm : -kNoTerm};
+  const uint32_t mh = (hi & 0xFFFFFu) | 0x100000u;
+  const int h = (int)((mh << 6) | (lo >> 26)), l = (int)(lo & 0x3FFFFFFu);
+  return (int)hi < 0 ? BetaFix{-h, -l, e} : BetaFix{h, l, e};
+}
+
+// a + b c, signed 32 x 32 bits into 64
+__device__ __forceinline__ long long madw(int b, int c, long long a) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a) : "r"(b), "r"(c));
+  return a;
+}
+// logical right shift that gives 0 from 32 on (the C operator does not define it)
+__device__ __forceinline__ uint32_t shr_clamp(uint32_t v, uint32_t n) {
+  asm("shr.u32 %0, %0, %1;" : "+r"(v) : "r"(n));
+  return v;
+}
+
+// Biased FP64 exponent of x and, left-aligned at bit 63 of (ah, al), its mantissa with the leading
+// bit; odd: neither a normal number nor zero.
+__device__ __forceinline__ void split_x(double x, int &e, bool &zero, bool &odd, uint32_t &ah, uint32_t &al, int &sgn) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  e = (int)((hi >> 20) & 0x7FFu);
+  zero = ((hi << 1) | lo) == 0u;
+  odd = (uint32_t)(e - 1) >= 2046u && !zero;
+  const uint32_t mh = (hi & 0xFFFFFu) | 0x100000u;
+  ah = __funnelshift_l(lo, mh, 11);
+  al = lo << 11;
+  sgn = ((int)hi >> 31) | 1;
+}
+__device__ __forceinline__ void split_x(float x, int &e, bool &zero, bool &odd, uint32_t &ah, uint32_t &al, int &sgn) {
+  const uint32_t u = __float_as_uint(x);
+  const int e8 = (int)((u >> 23) & 0xFFu);
+  zero = (u << 1) == 0u;
+  odd = (uint32_t)(e8 - 1) >= 254u && !zero;
+  e = e8 + 896;
+  ah = (u << 8) | 0x80000000u;
+  al = 0u;
+  sgn = ((int)u >> 31) | 1;
+}
+
+// (p3 2^78 + p2 2^52 + p1 2^26 + p0) 2^(F - 2133), rounded to nearest; 1200 <= F <= 3000, |total| < 2^99
+__device__ __forceinline__ double dot_total(uint32_t p0, uint32_t p1, uint32_t p2, int p3, int F) {
+  const long long top = ((long long)p3 << 26) + (long long)p2;                             // units of 2^52
+  const unsigned long long low = ((unsigned long long)p1 << 26) + (unsigned long long)p0;  // < 2^58
+  unsigned long long L = ((unsigned long long)top << 52) + low;
+  unsigned long long H = (unsigned long long)(top >> 12) + (L < low ? 1ull : 0ull);
+  const bool neg = (long long)H < 0;
+  if (neg) {
+    L = 0ull - L;
+    H = ~H + (L == 0ull ? 1ull : 0ull);
+  }
+  int pos = 127;  // of the leading bit
+  if (H == 0ull) {
+    H = L;
+    L = 0ull;
+    pos = 63;
+  }
+  if (H == 0ull) return 0.0;
+  const int n = __clzll((long long)H);
+  const unsigned long long m = n ? (H << n) | (L >> (64 - n)) : H;
+  // the 53 leading bits, rounded by the next one; a carry moves into the exponent
+  const unsigned long long bits = (m >> 11) + ((m >> 10) & 1ull) + ((unsigned long long)(uint32_t)(F - 2133 + 1022 + pos - n) << 52);
+  return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
+}
+
 // Tx = double (X F64 or U F64) or float (X F32, widened exactly).  VW = elements per lane load,
-// VMAX = lane loads per row (sized to d), RPW = rows per warp iteration.
-template <class Tx, int VW, int VMAX, int RPW>
-__global__ void __launch_bounds__(kGradThreads) k_grad_f64(const GradArgs a) {
-  __shared__ double sm[kWarps][512];
+// VMAX = lane loads per row (sized to d), RPW = rows per warp iteration.  BS: the parts of beta stay
+// in shared memory (16 columns per lane leave no registers for them).  Two CTAs of 8 warps fit on an
+// SM.  The rows of the next two groups are on their way meanwhile: every lane copies its own pieces
+// (cp.async) into its warp's two-stage ring in shared memory, which costs no registers.
+template <class Tx, int VW, int VMAX, int RPW, bool BS>
+__global__ void __launch_bounds__(kGradThreads, 2) k_grad_f64(const GradArgs a) {
+  extern __shared__ __align__(16) unsigned char ring_raw[];
+  __shared__ __align__(16) double sm[kWarps][512];
   if (a.check_done && a.st->done) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = (int64_t)blockIdx.x * kWarps + warp, nw = (int64_t)gridDim.x * kWarps;
@@ -153,19 +228,40 @@ __global__ void __launch_bounds__(kGradThreads) k_grad_f64(const GradArgs a) {
   const double *beta = a.beta_ring + (size_t)(a.st->iter % 3) * d;
   const Tx *X = static_cast<const Tx *>(a.X);
   const Tx *Y = static_cast<const Tx *>(a.Y);
-  double b[VMAX][VW], g[VMAX][VW];
+  constexpr int NB = BS ? 1 : VMAX * VW;
+  int rbh[NB], rbl[NB], rbe[NB];
+  // shared-memory form: (bh, bl) pairs, then the exponents, in lane order
+  int2 *sb = reinterpret_cast<int2 *>(&sm[0][0]);
+  int *se = reinterpret_cast<int *>(sb + 32 * VMAX * VW);
+  double g[VMAX][VW];
+  bool beta_odd = false;
 #pragma unroll
   for (int v = 0; v < VMAX; ++v)
 #pragma unroll
     for (int e = 0; e < VW; ++e) {
       const int col = (v * 32 + lane) * VW + e;
-      b[v][e] = col < d ? beta[col] : 0.0;
+      const BetaFix b = beta_fix(col < d ? beta[col] : 0.0);
+      beta_odd |= b.be == -kNoTerm;
+      if constexpr (BS) {
+        if (warp == 0) {
+          sb[(v * VW + e) * 32 + lane] = make_int2(b.bh, b.bl);
+          se[(v * VW + e) * 32 + lane] = b.be;
+        }
+      } else {
+        rbh[v * VW + e] = b.bh;
+        rbl[v * VW + e] = b.bl;
+        rbe[v * VW + e] = b.be;
+      }
       g[v][e] = 0.0;
     }
-  // The register tile wants one CTA per SM, so the rows of the next group are loaded (in their
-  // storage type) before the current group's FP64 arithmetic: its latency hides behind the FMAs.
-  Tx nx[RPW][VMAX][VW], ny[RPW];
-  auto load_rows = [&](int64_t i0) {
+  beta_odd = __any_sync(0xffffffffu, beta_odd);
+  if constexpr (BS) __syncthreads();
+  struct __align__(VW * sizeof(Tx)) Piece {
+    Tx e[VW];
+  };
+  // this warp's ring: stage, row, load, lane
+  Piece *ring = reinterpret_cast<Piece *>(ring_raw) + warp * (2 * RPW * VMAX * 32) + lane;
+  auto load_rows = [&](int64_t i0, int stage) {  // rows past the end and columns past d as zeros
 #pragma unroll
     for (int q = 0; q < RPW; ++q) {
       const int64_t i = i0 + q;
@@ -174,68 +270,136 @@ __global__ void __launch_bounds__(kGradThreads) k_grad_f64(const GradArgs a) {
 #pragma unroll
       for (int v = 0; v < VMAX; ++v) {
         const int col0 = (v * 32 + lane) * VW;
-        if (rv && col0 < d) Vec<Tx, VW>::load(row + col0, nx[q][v], true);
-        else {
-#pragma unroll
-          for (int e = 0; e < VW; ++e) nx[q][v][e] = Tx(0);
-        }
+        const bool in = rv && col0 < d;
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(ring + ((stage * RPW + q) * VMAX + v) * 32);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(dst), "l"(row + (in ? col0 : 0)),
+                     "n"((int)sizeof(Piece)), "r"(in ? (int)sizeof(Piece) : 0)
+                     : "memory");
       }
-      ny[q] = rv ? Y[i] : Tx(0);
     }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  auto load_y = [&](int64_t i0) -> Tx {  // lane q: row q's
+    return (lane < RPW && i0 + lane < a.nrows) ? Y[i0 + lane] : Tx(0);
   };
   const int64_t step = nw * RPW;
-  if (gw * RPW < a.nrows) load_rows(gw * RPW);
-  for (int64_t i0 = gw * RPW; i0 < a.nrows; i0 += step) {
-    double x[RPW][VMAX][VW];
-    double yv[RPW];
-    bool special = false;
+  load_rows(gw * RPW, 0);
+  load_rows(gw * RPW + step, 1);
+  Tx ny = load_y(gw * RPW);
+  int stage = 0;
+  for (int64_t i0 = gw * RPW; i0 < a.nrows; i0 += step, stage ^= 1) {
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    Tx x[RPW][VMAX][VW];
+    const double y = (double)ny;
+#pragma unroll
+    for (int q = 0; q < RPW; ++q)
+#pragma unroll
+      for (int v = 0; v < VMAX; ++v) {
+        const Piece t = ring[((stage * RPW + q) * VMAX + v) * 32];
+#pragma unroll
+        for (int e = 0; e < VW; ++e) x[q][v][e] = t.e[e];
+      }
+    load_rows(i0 + 2 * step, stage);
+    ny = load_y(i0 + step);
+    bool odd = false;
+    uint32_t p0 = 0u, p1 = 0u, p2 = 0u;
+    int p3 = 0, F = 1200;
 #pragma unroll
     for (int q = 0; q < RPW; ++q) {
+      int f[VMAX][VW], fmax = kNoTerm;
 #pragma unroll
       for (int v = 0; v < VMAX; ++v)
 #pragma unroll
-        for (int e = 0; e < VW; ++e)
-          x[q][v][e] = ((v * 32 + lane) * VW + e < d) ? widen(nx[q][v][e], special) : 0.0;
-      yv[q] = widen(ny[q], special);
+        for (int e = 0; e < VW; ++e) {
+          int ex, sgn;
+          bool zero, od;
+          uint32_t ah, al;
+          split_x(x[q][v][e], ex, zero, od, ah, al, sgn);
+          odd |= od;
+          const int be = BS ? se[(v * VW + e) * 32 + lane] : rbe[BS ? 0 : v * VW + e];
+          f[v][e] = zero ? kNoTerm : ex + be;
+          fmax = max(fmax, f[v][e]);
+        }
+      fmax = __reduce_max_sync(0xffffffffu, fmax);
+      long long sh = 0, s1 = 0, s2 = 0;
+#pragma unroll
+      for (int v = 0; v < VMAX; ++v)
+#pragma unroll
+        for (int e = 0; e < VW; ++e) {
+          int ex, sgn;
+          bool zero, od;
+          uint32_t ah, al;
+          split_x(x[q][v][e], ex, zero, od, ah, al, sgn);
+          const uint32_t t = (uint32_t)(fmax - f[v][e]) + 1u;  // right shift of (ah, al)
+          const int zh = (int)shr_clamp(ah, t) * sgn;
+          const int zl = (int)shr_clamp(__funnelshift_rc(al, ah, t), (uint32_t)max((int)t - 31, 1)) * sgn;
+          int2 b;
+          if constexpr (BS) b = sb[(v * VW + e) * 32 + lane];
+          else b = make_int2(rbh[v * VW + e], rbl[v * VW + e]);
+          sh = madw(zh, b.x, sh);
+          s1 = madw(zl, b.x, s1);
+          s2 = madw(zh, b.y, s2);
+        }
+      // sh 2^31 + s1 + s2 2^5, in 96 bits
+      const uint32_t hl = (uint32_t)sh, hh = (uint32_t)(sh >> 32);
+      uint32_t w0 = hl << 31, w1 = __funnelshift_l(hl, hh, 31), w2 = (uint32_t)((int)hh >> 1);
+      const uint32_t ml = (uint32_t)s2, mh = (uint32_t)(s2 >> 32);
+      asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+          : "+&r"(w0), "+&r"(w1), "+r"(w2)
+          : "r"((uint32_t)s1), "r"((uint32_t)(s1 >> 32)), "r"((uint32_t)(s1 >> 63)));
+      asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+          : "+&r"(w0), "+&r"(w1), "+r"(w2)
+          : "r"(ml << 5), "r"(__funnelshift_l(ml, mh, 5)), "r"((uint32_t)((int)mh >> 27)));
+      // 26-bit pieces (the top one signed), each summed over the lanes; lane q keeps row q's
+      const uint32_t q0 = __reduce_add_sync(0xffffffffu, w0 & 0x3FFFFFFu);
+      const uint32_t q1 = __reduce_add_sync(0xffffffffu, __funnelshift_r(w0, w1, 26) & 0x3FFFFFFu);
+      const uint32_t q2 = __reduce_add_sync(0xffffffffu, __funnelshift_r(w1, w2, 20) & 0x3FFFFFFu);
+      const int q3 = __reduce_add_sync(0xffffffffu, (int)w2 >> 14);
+      if (lane == q) { p0 = q0; p1 = q1; p2 = q2; p3 = q3; F = fmax; }
     }
-    if (i0 + step < a.nrows) load_rows(i0 + step);
-    if constexpr (sizeof(Tx) == 4) {
-      // a denormal, infinity or NaN among these rows (warp-uniform, rare): convert them again
-      if (__any_sync(0xffffffffu, special)) {
+    const bool rv = lane < RPW && i0 + lane < a.nrows;
+    odd = __any_sync(0xffffffffu, odd);
+    double r[RPW];
+    if (!beta_odd && !odd && !__any_sync(0xffffffffu, rv && (uint32_t)(F - 1200) > 1800u)) {
+      const double rl = rv ? y - dot_total(p0, p1, p2, p3, F) : 0.0;
 #pragma unroll
-        for (int q = 0; q < RPW; ++q) {
-          const int64_t i = i0 + q;
-          const bool rv = i < a.nrows;
-          const Tx *row = X + (rv ? i : 0) * a.ldx;
+      for (int q = 0; q < RPW; ++q) r[q] = __shfl_sync(0xffffffffu, rl, q);
+    } else {
+      double t[RPW];
 #pragma unroll
-          for (int v = 0; v < VMAX; ++v) {
-            const int col0 = (v * 32 + lane) * VW;
-#pragma unroll
-            for (int e = 0; e < VW; ++e) x[q][v][e] = (rv && col0 + e < d) ? (double)row[col0 + e] : 0.0;
-          }
-          yv[q] = rv ? (double)Y[i] : 0.0;
+      for (int q = 0; q < RPW; ++q) {
+        t[q] = 0.0;
+        const int64_t i = i0 + q;
+#pragma unroll 1
+        for (int v = 0; v < VMAX * VW; ++v) {
+          const int col = ((v / VW) * 32 + lane) * VW + v % VW;
+          if (col < d && i < a.nrows) t[q] = fma((double)X[i * a.ldx + col], beta[col], t[q]);
         }
       }
+      warp_sum_rows<RPW>(t, lane);
+#pragma unroll
+      for (int q = 0; q < RPW; ++q) r[q] = __shfl_sync(0xffffffffu, y, q) - t[q];
     }
-    double s[RPW];
+    // rows past the end are zero rows: x = 0 adds nothing
+    if (sizeof(Tx) == 4 && odd) {  // rare: values the integer widening does not take
 #pragma unroll
-    for (int q = 0; q < RPW; ++q) {
-      s[q] = 0.0;
+      for (int q = 0; q < RPW; ++q)
 #pragma unroll
-      for (int v = 0; v < VMAX; ++v)
+        for (int v = 0; v < VMAX; ++v)
 #pragma unroll
-        for (int e = 0; e < VW; ++e) s[q] = fma(x[q][v][e], b[v][e], s[q]);
-    }
-    warp_sum_rows<RPW>(s, lane);
+          for (int e = 0; e < VW; ++e) g[v][e] = fma((double)x[q][v][e], r[q], g[v][e]);
+    } else {
+      bool special = false;
 #pragma unroll
-    for (int q = 0; q < RPW; ++q) {
-      const double r = yv[q] - s[q];  // rows past the end are zero rows: x = 0 adds nothing
+      for (int q = 0; q < RPW; ++q)
 #pragma unroll
-      for (int v = 0; v < VMAX; ++v)
+        for (int v = 0; v < VMAX; ++v)
 #pragma unroll
-        for (int e = 0; e < VW; ++e) g[v][e] = fma(x[q][v][e], r, g[v][e]);
+          for (int e = 0; e < VW; ++e) g[v][e] = fma(widen(x[q][v][e], special), r[q], g[v][e]);
     }
   }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  if constexpr (BS) __syncthreads();  // the parts of beta share the array with the partials
 #pragma unroll
   for (int v = 0; v < VMAX; ++v)
 #pragma unroll
@@ -755,18 +919,32 @@ cudaError_t launch1(K kern, int nblk, const GradArgs &a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// FP64 kernel with its register tile sized to d (lane loads per row) and 4 rows per warp
-// iteration (2 for the widest tiles, whose rows take 32 doubles per lane)
+// FP64 kernel with its register tile sized to d (columns per lane) and several rows per warp
+// iteration (fewer as the rows widen)
+#define SLSE_GRAD64_VARIANTS(Tx, VW, F)                                              \
+  F(1, 4, (k_grad_f64<Tx, VW, 1, 4, false>)) F(2, 4, (k_grad_f64<Tx, VW, 2, 4, false>)) \
+  F(3, (VW == 1 ? 4 : 2), (k_grad_f64<Tx, VW, 3, (VW == 1 ? 4 : 2), false>))            \
+  F(4, (VW == 1 ? 4 : 2), (k_grad_f64<Tx, VW, 4, (VW == 1 ? 4 : 2), false>))            \
+  F(6, (VW == 1 ? 2 : 1), (k_grad_f64<Tx, VW, 6, (VW == 1 ? 2 : 1), (VW == 2)>))        \
+  F(8, (VW == 1 ? 2 : 1), (k_grad_f64<Tx, VW, 8, (VW == 1 ? 2 : 1), (VW == 2)>))
+#define SLSE_GRAD64_WIDE(Tx, V) (k_grad_f64<Tx, 1, V, 1, true>)
 template <class Tx, int VW>
 cudaError_t launch_f64(int d, int nblk, const GradArgs &a, cudaStream_t s) {
   constexpr int per = 32 * VW;
-  if (d <= per) return launch1(k_grad_f64<Tx, VW, 1, 4>, nblk, a, s);
-  if (d <= 2 * per) return launch1(k_grad_f64<Tx, VW, 2, 4>, nblk, a, s);
-  if (d <= 4 * per) return launch1(k_grad_f64<Tx, VW, 4, 4>, nblk, a, s);
-  if (d <= 8 * per) return launch1(k_grad_f64<Tx, VW, 8, 2>, nblk, a, s);
+  auto go = [&](auto kern, size_t row_bytes, int rows) -> cudaError_t {
+    const size_t smem = (size_t)kWarps * 2 * rows * row_bytes;  // at most 64 KB
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<nblk, kGradThreads, smem, s>>>(a);
+    return cudaGetLastError();
+  };
+#define SLSE_GRAD64_CASE(V, R, K) if (d <= V * per) return go(K, V * per * sizeof(Tx), R);
+  SLSE_GRAD64_VARIANTS(Tx, VW, SLSE_GRAD64_CASE)
   if constexpr (VW == 1) {
-    if (d <= 16 * per) return launch1(k_grad_f64<Tx, VW, 16, 2>, nblk, a, s);
+    if (d <= 12 * per) return go(SLSE_GRAD64_WIDE(Tx, 12), 12 * per * sizeof(Tx), 1);
+    if (d <= 16 * per) return go(SLSE_GRAD64_WIDE(Tx, 16), 16 * per * sizeof(Tx), 1);
   }
+#undef SLSE_GRAD64_CASE
   return cudaErrorInvalidValue;
 }
 
@@ -823,16 +1001,12 @@ cudaError_t launch_grad(int mode, int xdtype, const void *X, int64_t ldx, const 
 cudaError_t preload_grad_kernels() {
   // every kernel launch_grad (modes GM_F64 and GM_MIXED) and launch_reduce can pick
   const void *k[] = {
-      (const void *)k_grad_f64<double, 2, 1, 4>, (const void *)k_grad_f64<double, 2, 2, 4>,
-      (const void *)k_grad_f64<double, 2, 4, 4>, (const void *)k_grad_f64<double, 2, 8, 2>,
-      (const void *)k_grad_f64<double, 1, 1, 4>, (const void *)k_grad_f64<double, 1, 2, 4>,
-      (const void *)k_grad_f64<double, 1, 4, 4>, (const void *)k_grad_f64<double, 1, 8, 2>,
-      (const void *)k_grad_f64<double, 1, 16, 2>,
-      (const void *)k_grad_f64<float, 2, 1, 4>,  (const void *)k_grad_f64<float, 2, 2, 4>,
-      (const void *)k_grad_f64<float, 2, 4, 4>,  (const void *)k_grad_f64<float, 2, 8, 2>,
-      (const void *)k_grad_f64<float, 1, 1, 4>,  (const void *)k_grad_f64<float, 1, 2, 4>,
-      (const void *)k_grad_f64<float, 1, 4, 4>,  (const void *)k_grad_f64<float, 1, 8, 2>,
-      (const void *)k_grad_f64<float, 1, 16, 2>,
+#define SLSE_GRAD64_PTR(V, R, K) (const void *)K,
+      SLSE_GRAD64_VARIANTS(double, 2, SLSE_GRAD64_PTR) SLSE_GRAD64_VARIANTS(double, 1, SLSE_GRAD64_PTR)
+      SLSE_GRAD64_VARIANTS(float, 2, SLSE_GRAD64_PTR) SLSE_GRAD64_VARIANTS(float, 1, SLSE_GRAD64_PTR)
+      (const void *)SLSE_GRAD64_WIDE(double, 12), (const void *)SLSE_GRAD64_WIDE(double, 16),
+      (const void *)SLSE_GRAD64_WIDE(float, 12), (const void *)SLSE_GRAD64_WIDE(float, 16),
+#undef SLSE_GRAD64_PTR
       (const void *)k_grad_mixed<1, 16, 1, 1>,   (const void *)k_grad_mixed<4, 1, 1, 8>,
       (const void *)k_grad_mixed<4, 2, 1, 4>,    (const void *)k_grad_mixed<4, 4, 1, 2>,
       (const void *)k_grad_mixed<1, 16, 0, 1>,   (const void *)k_grad_mixed<4, 1, 0, 8>,
