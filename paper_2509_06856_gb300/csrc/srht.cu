@@ -41,6 +41,14 @@ namespace cg = cooperative_groups;
 namespace slse {
 namespace {
 
+// The intermediate W is stored in blocks of 2^kWBlock rows k2 of one j1: row (j1, k2) at
+// ((k2 >> kWBlock) n1 + j1) 2^kWBlock + k2 mod 2^kWBlock.  A pass-1 group writes
+// 2^kWBlock rows at a time and a pass-2 group's rows lie closer together than at the stride n2 of
+// plain row order, which helps the writes more than it costs the reads (bench shape, tensor-core
+// passes 1 + 2: plain order 3.38 + 1.45 ms, 8 rows 3.00 + 1.49, 32 rows 3.01 + 1.68, 128 rows 3.01 +
+// 2.14).  W^T W, which the Gram build takes from W, does not depend on the order of its rows.
+constexpr int kWBlock = 3;
+
 // Output tag for the FP8 form of the sketch: E4M3 values with one power-of-two scale per
 // 32-column block of a row (scale byte = exponent + 127); the rows' Y values stay BF16.
 struct mx8 {};
@@ -235,7 +243,7 @@ __global__ void __launch_bounds__(NT, MINB) k_group(const GroupArgs a) {
   // output scale; 0 for padding rows)
   const Ts scale = (Ts)a.scale;
   for (int l = threadIdx.x; l < M; l += NT) {
-    const int64_t j = (rho0 + l) * a.istride + g * a.igstride;
+    const int64_t j = in_row(a, rho0 + l, g);
     int64_t src = j;
     Ts mul = scale;
     if (a.Psd) {
@@ -258,7 +266,7 @@ __global__ void __launch_bounds__(NT, MINB) k_group(const GroupArgs a) {
       if (e < M) {
         const int q = e / MQ, lq = e % MQ;
         const int64_t kappa = (int64_t)q * M + rank * MQ + lq;
-        pos_reg[k] = __ldg(a.pos + kappa * a.ostride + g * a.ogstride);
+        pos_reg[k] = __ldg(a.pos + out_row(a, kappa, g));
       }
     }
   }
@@ -406,7 +414,7 @@ __global__ void __launch_bounds__(NT, MINB) k_group(const GroupArgs a) {
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
       const int64_t kappa = (int64_t)q * M + l;
-      const int64_t dst = a.pos ? (int64_t)s_dst[q * MQ + lq] : kappa * a.ostride + g * a.ogstride;
+      const int64_t dst = a.pos ? (int64_t)s_dst[q * MQ + lq] : out_row(a, kappa, g);
       if constexpr (std::is_same_v<Tout, mx8>) {
         // the 8 consecutive lanes with the same lq hold this row's 32-column block
         static_assert(VO == 4 && C == 32 && sizeof(Ts) == 4, "an FP8 block is one 32-column FP32 slab");
@@ -474,7 +482,7 @@ __global__ void __launch_bounds__(512) k_ycol(const GroupArgs a, int L) {
   const int64_t g = blockIdx.x;
   const Tin *in_y = static_cast<const Tin *>(a.in_y);
   for (int rho = threadIdx.x; rho < n; rho += blockDim.x) {
-    const int64_t j = rho * a.istride + g * a.igstride;
+    const int64_t j = in_row(a, rho, g);
     Ts v;
     if (a.Psd) {
       const int32_t c = __ldg(a.Psd + j);
@@ -498,7 +506,7 @@ __global__ void __launch_bounds__(512) k_ycol(const GroupArgs a, int L) {
   }
   Tout *out_y = static_cast<Tout *>(a.out_y);
   for (int kap = threadIdx.x; kap < n; kap += blockDim.x) {
-    const int64_t k = kap * a.ostride + g * a.ogstride;
+    const int64_t k = out_row(a, kap, g);
     const int64_t dst = a.pos ? (int64_t)__ldg(a.pos + k) : k;
     if (dst >= 0) store_cvt(out_y + dst, t[kap] * (Ts)a.scale);
   }
@@ -596,7 +604,24 @@ template <class Tin, class Ts, class Tout, int VA, int VB, int VO, int SLAB_BYTE
 cudaError_t launch_pass_t(const GroupArgs &a, int L, int64_t ngroups, cudaStream_t s) {
   constexpr int CP = SLAB_BYTES / (int)sizeof(Ts);
   cudaError_t e;
-  if constexpr (sizeof(Ts) == 8) {
+  // FP32 arithmetic, groups of 2^10 and 2^11 rows with 16-byte aligned rows: the tensor-core form
+  // (bench shape: passes 3.45 + 3.22 ms in the cluster form, 3.00 + 1.49 ms there; 2^12 rows would leave
+  // 16 columns of tensor memory, 32-byte row segments)
+  bool tc = false;
+  if constexpr (std::is_same_v<Tout, __nv_bfloat16>) {
+    auto ok16 = [](const void *p, int64_t ld, size_t eb) {
+      return reinterpret_cast<uintptr_t>(p) % 16 == 0 && ld % (int64_t)(16 / eb) == 0;
+    };
+    tc = (L == 10 || L == 11) && ok16(a.in, a.ldin, sizeof(Tin)) && a.ldin < (int64_t(1) << 30) &&
+         (std::is_same_v<Tin, float> ? a.Psd != nullptr : a.Psd == nullptr);
+    if (tc) {
+      GroupArgs b = a;
+      b.vec_out = ok16(a.out, a.ldout, 2) ? 1 : 0;
+      if ((e = launch_group_tc(b, std::is_same_v<Tin, float>, L, ngroups, s)) != cudaSuccess) return e;
+    }
+  }
+  if (tc) {
+  } else if constexpr (sizeof(Ts) == 8) {
     // FP64: from 2^8 rows a group on the integer pipe (srht64.cu: 2^10 rows, d = 200, 4.4 -> 1.7 ms
     // a pass); smaller groups (N' <= 2^15) do not fill its warps and take tens of microseconds
     switch (L) {
@@ -671,10 +696,11 @@ cudaError_t run_plan(const SrhtPlan &pl, const void *X, int64_t ldx, const void 
     return launch_small_t<Tin, Ts, Tout, C>(a, pl.logN, s);
   }
   const int64_t n1 = int64_t(1) << pl.log1, n2 = int64_t(1) << pl.log2;
+  const int blk = kWBlock < pl.log2 ? kWBlock : pl.log2;
   // pass 1: groups g = j1 (n1 of them), rows rho = j2 (n2 per group)
   a.istride = 1; a.igstride = n2;
   a.out = W; a.ldout = ldw; a.out_y = WY; a.pos = nullptr;
-  a.ostride = 1; a.ogstride = n2;
+  a.ostride = n1 << blk; a.ogstride = int64_t(1) << blk; a.oblk = blk;
   a.scale = 1.0;
   a.copy_out = copy_out;
   a.vec_out = vec_ok(W, ldw, sizeof(Tout), VO) ? 1 : 0;
@@ -691,11 +717,11 @@ cudaError_t run_plan(const SrhtPlan &pl, const void *X, int64_t ldx, const void 
   b.in = W; b.ldin = ldw; b.in_y = WY;
   b.vec_in = vec_ok(W, ldw, sizeof(Tout), VA) ? 1 : 0;
   b.vec_out = vec_ok(U, ldu, sizeof(Tout), VO) ? 1 : 0;
-  b.istride = n2; b.igstride = 1;
+  b.istride = int64_t(1) << blk; b.igstride = n1 << blk; b.iblk = blk;
   b.out = U; b.ldout = ldu; b.out_y = V; b.pos = pos;
   b.out_scale = Uscale; b.ld_scale = ld_scale;
   b.hat_out = hat; b.hat_row0 = hat_row0; b.hat_ld = hat_ld;
-  b.ostride = 1; b.ogstride = n1;  // pos is stored pass-2-major: entry (k2, k1) at k2 n1 + k1
+  b.ostride = 1; b.ogstride = n1; b.oblk = 0;  // pos is stored pass-2-major: entry (k2, k1) at k2 n1 + k1
   b.scale = scale;
   return pass2(b, pl.log1, n2, s);
 }

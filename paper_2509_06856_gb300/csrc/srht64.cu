@@ -171,7 +171,7 @@ __global__ void __launch_bounds__((1 << L) * C / kRows, 512 / ((1 << L) * C / kR
   const int64_t ldi = a.ldin * (int64_t)sizeof(Tin), ldo = a.ldout * (int64_t)sizeof(double);
 
   for (int l = t; l < M; l += NT) {
-    const int64_t j = l * a.istride + g * a.igstride;
+    const int64_t j = in_row(a, l, g);
     const int32_t v = a.Psd ? __ldg(a.Psd + j) : (int32_t)j;
     if constexpr (kOff) {
       const int64_t src = v < 0 ? (int64_t)(~v) : (int64_t)v;
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__((1 << L) * C / kRows, 512 / ((1 << L) * C / kR
   const int emax = max((int)(s_emax[c] >> 20), 1);
   // the output rows replace the input rows (every thread has read its own)
   for (int l = t; l < M; l += NT) {
-    const int64_t kg = l * a.ostride + g * a.ogstride;
+    const int64_t kg = out_row(a, l, g);
     const int64_t dst = a.pos ? (int64_t)__ldg(a.pos + kg) : kg;
     if constexpr (kOff) s_row[l] = dst < 0 ? -1 : dst * ldo;
     else s_row[l] = (int32_t)dst;

@@ -11,12 +11,16 @@ struct GroupArgs {
   const void *in_y;     // Y or WY
   int64_t N;            // gather mode: rows >= N are the zero padding
   const int32_t *Psd;   // non-null: gather mode (sign-folded permutation)
-  int64_t istride, igstride;  // input row j = rho * istride + g * igstride
+  // input row of element rho of group g: rho * istride + (g >> iblk) * igstride + (g mod 2^iblk)
+  int64_t istride, igstride;
+  int iblk;
   void *out;
   int64_t ldout;
   void *out_y;
   const int32_t *pos;   // non-null: output row = pos[k], skipped when < 0
-  int64_t ostride, ogstride;  // output index k = kappa * ostride + g * ogstride
+  // output index of element kappa: (kappa >> oblk) * ostride + (kappa mod 2^oblk) + g * ogstride
+  int64_t ostride, ogstride;
+  int oblk;
   int d;
   int nslab;
   int logq;
@@ -31,8 +35,20 @@ struct GroupArgs {
   unsigned *status;     // nullable: ST_TIMEOUT is raised here when a bounded wait gave up
 };
 
+__host__ __device__ __forceinline__ int64_t in_row(const GroupArgs &a, int64_t rho, int64_t g) {
+  return rho * a.istride + (g >> a.iblk) * a.igstride + (g & ((int64_t(1) << a.iblk) - 1));
+}
+__host__ __device__ __forceinline__ int64_t out_row(const GroupArgs &a, int64_t kappa, int64_t g) {
+  return (kappa >> a.oblk) * a.ostride + (kappa & ((int64_t(1) << a.oblk) - 1)) + g * a.ogstride;
+}
+
 // srht64.cu: the X columns of one FP64 pass over groups of 2^L rows (8 <= L <= 12) in 96-bit
 // fixed point.  Tin = double, or float for pass 1 on FP32 storage.
 template <class Tin> cudaError_t launch_group_fix(const GroupArgs &a, int L, int64_t ngroups, cudaStream_t s);
+
+// srht_tc.cu: the X columns of one mixed-precision pass over groups of 2^10 or 2^11 rows on the
+// tensor cores: FP32 rows gathered through Psd (pass 1) or BF16 rows (pass 2) in, BF16 rows out.
+// The rows read are 16-byte aligned (ldin a multiple of 4 FP32 or 8 BF16 elements).
+cudaError_t launch_group_tc(const GroupArgs &a, bool f32, int L, int64_t ngroups, cudaStream_t s);
 
 }  // namespace slse
