@@ -7,11 +7,12 @@
 // The normal-equation solve is the M-IHS iteration of the 2nd stage with the gradient
 // replaced by v - X^T X w, preconditioned by the H-hat^{-1} of the fit (paper Eqs. (7),
 // (8)), so it converges at the fit's rate: w+ = w + mu H^{-1}(v - X^T X w) + eta (w - w_prev).
-// Each iteration is one pass over X (the residual-gradient kernels with Y = 0).
+// Each iteration is one pass over X (the residual-gradient kernels with Y = 0) or, on the mixed path
+// in correction form (as in the fit's 2nd stage), a d x d product between exact passes.
 #include <cmath>
 #include <type_traits>
 
-#include "slse_internal.cuh"
+#include "host_res.cuh"
 
 namespace slse {
 namespace {
@@ -20,19 +21,13 @@ constexpr size_t kStateBytesA = 4096;
 
 inline size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
-__global__ void k_init_adj(DevState *st, int rebase) {
+__global__ void k_init_adj(DevState *st, int rebase, int dc) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     DevState z = {};
     z.rebase = rebase;
+    z.dc = dc;
     *st = z;
   }
-}
-
-// g <- v + g (g holds X^T (0 - X w) = -X^T X w); skipped once the stop flag is set.
-__global__ void k_add_rhs(double *g, const double *v, int d, const DevState *st) {
-  if (st->done) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < d) g[i] = v[i] + g[i];
 }
 
 // One warp per row: a = x.w, p = x.beta (FP32 inputs: compensated products and sums with
@@ -253,23 +248,16 @@ __global__ void __launch_bounds__(256, MINB) k_vjp_rows_f32v(const float *X, int
   }
 }
 
-// Pinned mailbox for the stop flag (one per host thread).
-struct MailboxA {
-  DevState *h = nullptr;
-  ~MailboxA() {
-    if (h) cudaFreeHost(h);
-  }
-  DevState *get() {
-    if (!h && cudaHostAlloc((void **)&h, 4 * sizeof(DevState), cudaHostAllocDefault) != cudaSuccess) h = nullptr;
-    return h;
-  }
-};
-thread_local MailboxA t_mbox;
-
 struct AdjLayout {
   int nblk;
-  size_t o_state, o_part, o_g, o_ring, o_b0, o_d32, o_r0, o_y0, total;
+  size_t o_state, o_part, o_g, o_ring, o_b0, o_d32, o_r0, o_y0, full;
+  bool dc;  // mixed path, correction form: the arrays below, behind those of the full form
+  GramPlan grp;
+  size_t o_g0, o_be, o_de, o_gb, o_gram, total;
 };
+
+// From this many elements of X on the backward solve takes the correction form (off).
+constexpr int64_t kAdjCorrection = INT64_MAX;
 
 AdjLayout adj_layout(const slse_problem *p, int prec, int nsm) {
   AdjLayout L{};
@@ -285,6 +273,16 @@ AdjLayout adj_layout(const slse_problem *p, int prec, int nsm) {
   L.o_d32 = take((size_t)d * 4);
   L.o_r0 = take(prec == SLSE_PREC_MIXED_BF16 ? (size_t)p->N * 4 : 0);
   L.o_y0 = take((size_t)p->N * (p->dtype == SLSE_F64 ? 8 : 4));
+  L.full = o;
+  L.dc = prec == SLSE_PREC_MIXED_BF16 && p->dtype == SLSE_F32 && p->N * d >= kAdjCorrection;
+  if (L.dc) {
+    L.grp = gram_plan(p->N, d, nsm > 0 ? nsm : 152);
+    L.o_g0 = take((size_t)d * 8);
+    L.o_be = take((size_t)d * 8);
+    L.o_de = take((size_t)d * 4);
+    L.o_gb = take((size_t)d * d * 8);
+    L.o_gram = take(L.grp.total);
+  }
   L.total = o;
   return L;
 }
@@ -344,9 +342,11 @@ extern "C" slse_status slse_solve_normal(const slse_problem *prob, const double 
       return SLSE_ENOMEM;
     }
     owned = true;
-  } else if (ws_bytes < L.total) {
+  } else if (ws_bytes < L.full) {
     return SLSE_ENOMEM;
   }
+  // a workspace without room for the Gram matrix keeps the full form
+  const bool dc = L.dc && sched->stage2 == SLSE_STAGE2_CORRECTION && (owned || ws_bytes >= L.total);
   struct Free {
     void *p;
     bool own;
@@ -367,21 +367,25 @@ extern "C" slse_status slse_solve_normal(const slse_problem *prob, const double 
   const int d = prob->d;
   const bool mixed = prec == SLSE_PREC_MIXED_BF16;
 
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  CKA(cudaEventCreate(&e0));
-  CKA(cudaEventCreate(&e1));
-  struct Ev {
-    cudaEvent_t a, b;
-    ~Ev() {
-      cudaEventDestroy(a);
-      cudaEventDestroy(b);
-    }
-  } evg{e0, e1};
+  double *g0 = dc ? reinterpret_cast<double *>(base + L.o_g0) : nullptr;
+  float *de = dc ? reinterpret_cast<float *>(base + L.o_de) : nullptr;
+  double *Gb = dc ? reinterpret_cast<double *>(base + L.o_gb) : nullptr;
+
+  Events E;
+  cudaEvent_t e0 = E.make(), e1 = E.make();
+  DevState *mb = host_res().mailbox();
+  volatile unsigned *word = host_res().stop_word();
+  if (!e0 || !e1 || !mb || !word) return SLSE_ECUDA;
   CKA(cudaEventRecord(e0, s));
-  k_init_adj<<<1, 32, 0, s>>>(st, mixed ? 1 : 0);
+  k_init_adj<<<1, 32, 0, s>>>(st, mixed ? 1 : 0, dc ? 1 : 0);
   CKA(cudaGetLastError());
   CKA(cudaMemsetAsync(ring, 0, (size_t)3 * d * 8, s));
   CKA(cudaMemsetAsync(y0, 0, (size_t)prob->N * (prob->dtype == SLSE_F64 ? 8 : 4), s));
+  int launches = 3;
+  if (dc) {
+    CKA(launch_gram(L.grp, static_cast<const float *>(prob->X), prob->ldx, Gb, &st->status, base + L.o_gram, s));
+    launches += gram_fp32_path(L.grp, static_cast<const float *>(prob->X), prob->ldx) ? 3 : 4;
+  }
 
   UpdateArgs ua{};
   ua.g = g; ua.Hinv = Hinv; ua.beta_ring = ring; ua.beta0 = b0; ua.delta32 = d32;
@@ -389,35 +393,25 @@ extern "C" slse_status slse_solve_normal(const slse_problem *prob, const double 
   const double rho = std::sqrt((double)d / (double)sched->r);
   ua.thr = sched->tol > 0.0 ? sched->tol * (1.0 - rho) / rho : 0.0;
   ua.stage2 = 1; ua.mixed = mixed ? 1 : 0; ua.check_done = 1;
-  DevState *mb = t_mbox.get();
-  if (!mb) return SLSE_ECUDA;
-  cudaEvent_t flag[2];
-  CKA(cudaEventCreateWithFlags(&flag[0], cudaEventDisableTiming));
-  CKA(cudaEventCreateWithFlags(&flag[1], cudaEventDisableTiming));
-  struct Ev2 {
-    cudaEvent_t *f;
-    ~Ev2() {
-      cudaEventDestroy(f[0]);
-      cudaEventDestroy(f[1]);
-    }
-  } evf{flag};
-  int launches = 3;
+  ua.beta_e = dc ? reinterpret_cast<double *>(base + L.o_be) : nullptr;
+  ua.delta_e = de;
+  correction_gains(rho, 0.02, ua.gain);
+  *word = 0u;
+  ua.mail = const_cast<unsigned *>(word);
   for (int k = 0; k < sched->T; ++k) {
     if (launch_grad(mixed ? GM_MIXED : GM_F64, prob->dtype, prob->X, prob->ldx, y0, prob->N, d, ring, st, d32, r0, b0,
                     part, L.nblk, 1, s) != cudaSuccess)
       return SLSE_ECUDA;
-    if (launch_reduce(part, L.nblk, d, 1.0, g, st, 1, s) != cudaSuccess) return SLSE_ECUDA;
-    k_add_rhs<<<(d + 255) / 256, 256, 0, s>>>(g, v, d, st);
-    CKA(cudaGetLastError());
+    // v + X^T (0 - X w), or the correction step's product
+    if (launch_reduce(part, L.nblk, d, 1.0, g, st, 1, s, g0, Gb, de, v) != cudaSuccess) return SLSE_ECUDA;
     ua.first = k == 0;
     if (launch_update(ua, st, s) != cudaSuccess) return SLSE_ECUDA;
-    launches += mixed ? 5 : 4;
-    // iteration k+1 is enqueued before the stop flag of iteration k is read back
-    CKA(cudaMemcpyAsync(&mb[k & 1], st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
-    CKA(cudaEventRecord(flag[k & 1], s));
+    launches += 3;
+    // iteration k+1 is enqueued before iteration k is awaited
     if (k > 0) {
-      CKA(cudaEventSynchronize(flag[(k - 1) & 1]));
-      if (((volatile DevState *)&mb[(k - 1) & 1])->done) break;
+      bool stopped = false;
+      CKA(wait_iterations(word, (unsigned)k, s, stopped));
+      if (stopped) break;
     }
   }
   if (launch_copy_beta(ring, st, d, w_out, s) != cudaSuccess) return SLSE_ECUDA;
@@ -428,7 +422,8 @@ extern "C" slse_status slse_solve_normal(const slse_problem *prob, const double 
   DevState fin{};
   fin.iter = fv->iter;
   fin.status = fv->status;
-  fin.rel_step = fv->rel_step;
+  fin.step2 = fv->step2;
+  fin.norm2 = fv->norm2;
   fin.rebases = fv->rebases;
   const slse_status status = from_bits(fin.status);
   if (report) {
@@ -437,7 +432,7 @@ extern "C" slse_status slse_solve_normal(const slse_problem *prob, const double 
     report->ms_total = ms;
     report->ms_stage2 = ms;
     report->iters_stage2 = fin.iter;
-    report->final_rel_step = fin.rel_step;
+    report->final_rel_step = rel_step(fin);
     report->rebases = fin.rebases;
     report->kernels = launches;
     report->status = status;

@@ -9,7 +9,7 @@
 #include <cstring>
 #include <vector>
 
-#include "slse_internal.cuh"
+#include "host_res.cuh"
 
 using namespace slse;
 
@@ -25,6 +25,15 @@ bool slse::is_host_pointer(const void *ptr) {
 
 namespace {
 std::atomic<long long> g_spin_limit{0};
+}
+void slse::correction_gains(double rho, double cost, double (&gain)[kMaxInner + 1]) {
+  for (int k = 0; k <= kMaxInner; ++k) {
+    const double g = std::pow(rho, 2.0 * (1.0 + cost * k));
+    gain[k] = g < 0.01 ? g : 0.01;
+  }
+}
+double slse::rel_step(const DevState &s) {
+  return s.norm2 > 0.0 ? std::sqrt(s.step2) / std::sqrt(s.norm2) : 0.0;
 }
 long long slse::debug_spin_limit() { return g_spin_limit.load(std::memory_order_relaxed); }
 
@@ -354,32 +363,6 @@ struct NvtxPhase {
   }
 };
 
-struct Events {
-  std::vector<cudaEvent_t> ev;
-  cudaEvent_t make() {
-    cudaEvent_t e = nullptr;
-    if (cudaEventCreate(&e) != cudaSuccess) return nullptr;
-    ev.push_back(e);
-    return e;
-  }
-  ~Events() {
-    for (auto e : ev) cudaEventDestroy(e);
-  }
-};
-
-// Pinned host mailbox for the stage-2 stop flag (one per host thread).
-struct Mailbox {
-  DevState *h = nullptr;
-  ~Mailbox() {
-    if (h) cudaFreeHost(h);
-  }
-  DevState *get() {
-    if (!h && cudaHostAlloc((void **)&h, 4 * sizeof(DevState), cudaHostAllocDefault) != cudaSuccess) h = nullptr;
-    return h;
-  }
-};
-thread_local Mailbox t_mailbox;
-
 float ms_between(cudaEvent_t a, cudaEvent_t b) {
   float ms = 0.f;
   if (a && b && cudaEventElapsedTime(&ms, a, b) != cudaSuccess) {
@@ -476,9 +459,9 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
   // is instead read by SRHT pass 1 straight from host memory (every row is gathered exactly
   // once there), and that pass also stores each row segment into the workspace copy: the
   // transfer over the host link and the pass are one step instead of two.
-  struct SideStream {
+  struct CopyStream {
     cudaStream_t h = nullptr;
-    ~SideStream() {
+    ~CopyStream() {
       if (h) cudaStreamDestroy(h);
     }
   } side;
@@ -582,22 +565,7 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
   // (free once the sketch is formed), so it is formed on a second stream beside the Hessian factor
   // and the 1st stage (memory- and latency-bound work beside a tensor-core product); the 2nd stage
   // waits for it
-  struct GramStream {
-    cudaStream_t h = nullptr, main = nullptr;
-    ~GramStream() {
-      if (!h) return;
-      // the caller's stream (on which a library-owned workspace is freed) waits for this one,
-      // also on an early return between the fork and the join
-      cudaEvent_t e = nullptr;
-      if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess) {
-        cudaEventRecord(e, h);
-        cudaStreamWaitEvent(main, e, 0);
-        cudaEventDestroy(e);
-      }
-      cudaStreamDestroy(h);
-    }
-  } gram_side;
-  gram_side.main = st;
+  SideStream gram_side;  // the caller's stream waits for it on every return
   double *Gb = L.dc ? reinterpret_cast<double *>(base + L.o_gb) : nullptr;
   unsigned *gram_status = L.dc ? reinterpret_cast<unsigned *>(base + L.o_gst) : nullptr;
   cudaEvent_t e_gram0 = nullptr, e_gram1 = nullptr;
@@ -605,7 +573,7 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
     e_gram0 = E.make();
     e_gram1 = E.make();
     if (!e_gram0 || !e_gram1) return SLSE_ECUDA;
-    CK(cudaStreamCreateWithFlags(&gram_side.h, cudaStreamNonBlocking));
+    CK(gram_side.open(false, st));
   }
   // The build is forked once the Hessian factor is formed: beside pass 2 (which also reads W) it
   // slowed the pass by half, and beside the Hessian factor's chain of short kernels it tripled the
@@ -634,25 +602,10 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
   // priority its pending CTAs were dispatched first, so the short kernels of the Hessian factor
   // waited for most of the build (0.86 ms became 4.3 ms).  The caller's stream joins it after the
   // 2nd stage (and waits for it on every return).
-  struct PrioStream {
-    cudaStream_t h = nullptr, user = nullptr;
-    ~PrioStream() {
-      if (!h) return;
-      cudaEvent_t e = nullptr;
-      if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess) {
-        cudaEventRecord(e, h);
-        cudaStreamWaitEvent(user, e, 0);
-        cudaEventDestroy(e);
-      }
-      cudaStreamDestroy(h);
-    }
-  } prio;
-  prio.user = st;
+  SideStream prio;
   const cudaStream_t user_st = st;
   if (gram_side.h) {
-    int least = 0, greatest = 0;
-    CK(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-    CK(cudaStreamCreateWithPriority(&prio.h, cudaStreamNonBlocking, greatest));
+    CK(prio.open(true, st));
     CK(cudaStreamWaitEvent(prio.h, e_sketch, 0));
     st = prio.h;
   }
@@ -684,7 +637,7 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
     CK(launch_gram_sweep(Uh, ldh, h0, s.r, d, hat_scale2, Hinv, base + L.o_chol, dst, st));
     const int nb = (d + 31) / 32;
     kernels += 3 + 2 * nb;
-    DevState *mb = t_mailbox.get();
+    DevState *mb = host_res().mailbox();
     if (!mb) return SLSE_ECUDA;
     CK(cudaMemcpyAsync(&mb[3], dst, sizeof(DevState), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -745,8 +698,10 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
   CK(cudaEventRecord(e_s1, st));
   phase.set("slse_fit: stage 2");
   // a8 stage 2: full-data M-IHS steps until the relative step is small or T is reached.
-  // Iteration k+1 is enqueued before the stop flag of iteration k is read back; its
-  // kernels return at once when the flag is already set.
+  // Iteration k+1 is enqueued before iteration k is awaited; its kernels return at once when the
+  // stop flag is already set.  The update kernel writes iterations and flag to pinned host memory,
+  // which the host polls: a copy and an event per step, two more events created and five launches
+  // made this loop host-bound (small fits 44 -> 29 us a step).
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> e_grad;
   // correction form: the Gram matrix G_b of the BF16 copy of X (formed once, here), g(beta_e)
   // beside the gradient, the iterate beta_e of the last exact pass and fl32(beta - beta_e)
@@ -755,8 +710,6 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
   ua.hist_base = t;
   ua.beta_e = L.dc ? reinterpret_cast<double *>(base + L.o_be) : nullptr;
   ua.delta_e = de;
-  // a correction step (a d x d product and the update) costs a small fraction of a pass over X
-  ua.inner_cost = 0.02;
   // G_b is first read by the 2nd stage's second step (its first pass is exact), so the main stream
   // waits for the side stream only there: the Gram build also overlaps that pass.  The wait is
   // enqueued before the call's last synchronisation in every case.
@@ -774,37 +727,38 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
     k_set_stage2<<<1, 32, 0, st>>>(dst, mixed ? 1 : 0, L.dc ? 1 : 0);
     CK(cudaGetLastError());
     ++kernels;
-    DevState *mb = t_mailbox.get();
+    DevState *mb = host_res().mailbox();
     if (!mb) return SLSE_ECUDA;
     const double rho = std::sqrt((double)d / (double)s.r);
     const double thr = s.tol > 0.0 ? s.tol * (1.0 - rho) / rho : 0.0;
-    ua.rho = rho;
+    // a correction step (a d x d product and the update) costs a small fraction of a pass over X
+    correction_gains(rho, 0.02, ua.gain);
     const int nb = L.nblk;
-    cudaEvent_t e_flag[2] = {E.make(), E.make()};
-    if (!e_flag[0] || !e_flag[1]) return SLSE_ECUDA;
+    volatile unsigned *word = host_res().stop_word();
+    *word = (unsigned)t << 1;
+    ua.mail = const_cast<unsigned *>(word);
     for (int k = 0; t + k < T; ++k) {
       cudaEvent_t g0e = E.make(), g1 = E.make();
       if (!g0e || !g1) return SLSE_ECUDA;
       if (k == 1) CK(join_gram());
       CK(cudaEventRecord(g0e, st));
       // correction form: a pass over X (exact) or a correction step g = g(beta_e) - G_b (beta - beta_e),
-      // as the device state selects; the kernels of the other kind return at once
+      // as the device state selects (the pass returns at once on a correction step)
       CK(launch_grad(mixed ? GM_MIXED : GM_F64, p->dtype, p->X, p->ldx, p->Y, p->N, d, ring, dst, d32, r0, b0,
                      part, nb, 1, st));
-      if (L.dc) CK(launch_gram_step(Gb, de, g0, g, d, dst, st));
-      CK(cudaEventRecord(g1, st));
+      if (!L.dc) CK(cudaEventRecord(g1, st));
+      CK(launch_reduce(part, nb, d, 1.0, g, dst, 1, st, g0, Gb, de));  // or the correction step's product
+      if (L.dc) CK(cudaEventRecord(g1, st));
       e_grad.emplace_back(g0e, g1);
-      CK(launch_reduce(part, nb, d, 1.0, g, dst, 1, st, g0));
       ua.first = (k == 0 && s.momentum_reset) || (t + k) == 0;
       ua.stage2 = 1; ua.thr = thr; ua.mixed = mixed ? 1 : 0; ua.check_done = 1;
       CK(launch_update(ua, dst, st));
-      kernels += L.dc ? 5 : (mixed ? 4 : 3);
+      kernels += 3;
       CK(mark_iter(t + k));
-      CK(cudaMemcpyAsync(&mb[k & 1], dst, sizeof(DevState), cudaMemcpyDeviceToHost, st));
-      CK(cudaEventRecord(e_flag[k & 1], st));
       if (k > 0) {
-        CK(cudaEventSynchronize(e_flag[(k - 1) & 1]));
-        if (((volatile DevState *)&mb[(k - 1) & 1])->done) break;
+        bool stopped = false;
+        CK(wait_iterations(word, (unsigned)(t + k), st, stopped));
+        if (stopped) break;
       }
     }
   }
@@ -818,7 +772,7 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
   }
   CK(launch_copy_beta(ring, dst, d, outb, st));
   ++kernels;
-  DevState *mb = t_mailbox.get();
+  DevState *mb = host_res().mailbox();
   if (!mb) return SLSE_ECUDA;
   CK(cudaMemcpyAsync(&mb[2], dst, sizeof(DevState), cudaMemcpyDeviceToHost, st));
   CK(cudaEventRecord(e_end, st));
@@ -874,7 +828,7 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
     RP->kernels = kernels;
     RP->iters_stage1 = t1;
     RP->iters_stage2 = fin.iter - t1;
-    RP->final_rel_step = fin.rel_step;
+    RP->final_rel_step = rel_step(fin);
     RP->rebases = fin.rebases;
     const double bx = p->dtype == SLSE_F64 ? 8.0 : 4.0, bu = (double)elem_bytes_u(s.prec);
     double bytes = 0.0;

@@ -25,7 +25,7 @@
 // Correction form of the mixed 2nd stage: exact passes stream X (the re-basing pass above or the
 // plain FP32 pass); the reduction keeps their gradient g(beta_e).  The steps between exact ones
 // use g(beta) = g(beta_e) - G_b (beta - beta_e) with the Gram matrix G_b = Xb^T Xb of the BF16 copy
-// Xb of X, formed once on the tensor cores (gram.cu): a d x d product (k_gram_step) instead of a
+// Xb of X, formed once on the tensor cores (gram.cu): a d x d product (in k_reduce) instead of a
 // pass over X.  The update kernel schedules the next exact pass (a step below 1/100 of the first
 // step after the last exact pass, a step above it, or one that meets the stopping test), makes it
 // a re-basing pass only when the drift from beta_0 exceeds 2^-10 ||beta||, stops only on an exact
@@ -537,15 +537,11 @@ __global__ void __launch_bounds__(kGradThreads) k_grad_bf16s(const GradArgs a) {
 
 // ---------------------------------------------------------------- mixed 2nd stage (X F32)
 // REBASE = 1: error-free residual against beta (FP64) and r0 written; REBASE = 0:
-// residual r0 - x . delta32.  The host launches both; the one whose mode does not
-// match st->rebase returns at once.  The two-word accumulators (hi, lo) of each
-// warp live in shared memory (float2 per column), folded every kFlushRows rows.
+// residual r0 - x . delta32.  The device state (st->rebase) selects the one that runs.  The
+// two-word accumulators (hi, lo) of each warp live in shared memory (float2 per column), folded
+// every kFlushRows rows.
 template <int VW, int VMAX, int REBASE, int RPW>
-__global__ void __launch_bounds__(kGradThreads, 2) k_grad_mixed(const GradArgs a) {
-  __shared__ __align__(16) double sm[kWarps][512];
-  if (a.check_done && a.st->done) return;
-  if ((a.st->rebase != 0) != (REBASE != 0)) return;
-  if (!REBASE && a.st->dc && a.st->bfnext) return;  // correction form: a correction step, not a pass
+__device__ __forceinline__ void grad_mixed_body(const GradArgs &a, double (*sm)[512]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = (int64_t)blockIdx.x * kWarps + warp, nw = (int64_t)gridDim.x * kWarps;
   const int d = a.d;
@@ -688,35 +684,88 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_grad_mixed(const GradArgs a
   cta_partial(sm, d, a.partials + (size_t)blockIdx.x * d);
 }
 
-// ---------------------------------------------------------------- reduction and update
-__global__ void k_reduce(const double *partials, int nblk, int d, double scale, double *g, const DevState *st,
-                         int check_done, double *g0) {
-  __shared__ double sm[8][33];
-  if (check_done && st->done) return;
-  if (g0 && st->dc && st->bfnext && !st->rebase) return;  // a correction step writes g itself
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c = blockIdx.x * 32 + lane;
-  // four independent sums over CTAs warp, warp + 8, ... (loads overlap), combined in a fixed order
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-  if (c < d) {
-    int b = warp;
-    for (; b + 24 < nblk; b += 32) {
-      s0 += partials[(size_t)b * d + c];
-      s1 += partials[(size_t)(b + 8) * d + c];
-      s2 += partials[(size_t)(b + 16) * d + c];
-      s3 += partials[(size_t)(b + 24) * d + c];
-    }
-    for (; b < nblk; b += 8) s0 += partials[(size_t)b * d + c];
+// One launch for both residual forms: a launch that returns at once still cost its start (1.4 us) and
+// the host the call.
+template <int VW, int VMAX, int RPW>
+__global__ void __launch_bounds__(kGradThreads, 2) k_grad_mixed(const GradArgs a) {
+  __shared__ __align__(16) double sm[kWarps][512];
+  if (a.check_done && a.st->done) return;
+  if (a.st->rebase) {
+    grad_mixed_body<VW, VMAX, 1, RPW>(a, sm);
+  } else {
+    if (a.st->dc && a.st->bfnext) return;  // correction form: a correction step, not a pass
+    grad_mixed_body<VW, VMAX, 0, RPW>(a, sm);
   }
-  sm[warp][lane] = (s0 + s1) + (s2 + s3);
-  __syncthreads();
-  if (warp == 0 && c < d) {
-    double t = 0.0;
+}
+
+// ---------------------------------------------------------------- reduction and update
+struct ReduceArgs {
+  const double *partials;
+  int nblk, d;
+  double scale;
+  double *g;
+  const DevState *st;
+  int check_done;
+  double *g0;            // correction form: g(beta_e)
+  const double *Gb;      // correction form: the Gram matrix and fl32(beta - beta_e)
+  const float *delta_e;
+  const double *rhs;     // added to the gradient of a pass
+};
+
+// g of this iteration, eight columns per CTA: the sum of the per-CTA partials of a pass, or, on a
+// correction step, g0 - G_b delta_e (one warp per row of G_b).  Latency: every thread has all its
+// partials (at most 12 per round) on their way at once, and the sums are short trees (an FP64 add
+// takes 64 cycles on this part, a double shuffle and add 101).  5.1 -> 2.9 us at d = 37 against sums in
+// four chains; the correction step's product used to be a launch of its own (2.6 us).
+__global__ void __launch_bounds__(256) k_reduce(const ReduceArgs a) {
+  __shared__ double sm[8][8];
+  const DevState *st = a.st;
+  if (a.check_done && st->done) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, d = a.d;
+  if (a.g0 && st->dc && st->bfnext && !st->rebase) {
+    const int i = blockIdx.x * 8 + warp;
+    if (i >= d) return;
+    const double *row = a.Gb + (size_t)i * d;
+    // four independent FP64 sums, fixed order
+    double h0 = 0.0, h1 = 0.0, h2 = 0.0, h3 = 0.0;
+    int k = lane;
+    for (; k + 96 < d; k += 128) {
+      h0 = fma(row[k], (double)a.delta_e[k], h0);
+      h1 = fma(row[k + 32], (double)a.delta_e[k + 32], h1);
+      h2 = fma(row[k + 64], (double)a.delta_e[k + 64], h2);
+      h3 = fma(row[k + 96], (double)a.delta_e[k + 96], h3);
+    }
+    for (; k < d; k += 32) h0 = fma(row[k], (double)a.delta_e[k], h0);
+    const double h = warp_sum((h0 + h1) + (h2 + h3));
+    if (lane == 0) a.g[i] = a.g0[i] - h;
+    return;
+  }
+  const int c = blockIdx.x * 8 + (lane & 7), b0 = threadIdx.x >> 3;  // column; partials b0, b0 + 32, ...
+  double s = 0.0;
+  if (c < d) {
+    for (int base = b0; base < a.nblk; base += 32 * 12) {
+      double v[12];
 #pragma unroll
-    for (int w = 0; w < 8; ++w) t += sm[w][lane];
-    const double v = scale * t;
-    if (g0) g0[c] = v;  // exact pass: keep g(beta_e)
-    g[c] = v;
+      for (int k = 0; k < 12; ++k) v[k] = base + 32 * k < a.nblk ? a.partials[(size_t)(base + 32 * k) * d + c] : 0.0;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) v[k] += v[k + 6];
+      s += ((v[0] + v[1]) + (v[2] + v[3])) + (v[4] + v[5]);
+    }
+  }
+  s += __shfl_xor_sync(0xffffffffu, s, 8);
+  s += __shfl_xor_sync(0xffffffffu, s, 16);
+  if (lane < 8) sm[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0) {
+    double t = sm[lane >> 3][lane & 7] + sm[(lane >> 3) + 4][lane & 7];
+    t += __shfl_xor_sync(0xffffffffu, t, 8);
+    t += __shfl_xor_sync(0xffffffffu, t, 16);
+    if (lane < 8 && c < d) {
+      double v = a.scale * t;
+      if (a.rhs) v += a.rhs[c];
+      if (a.g0) a.g0[c] = v;  // exact pass: keep g(beta_e)
+      a.g[c] = v;
+    }
   }
 }
 
@@ -728,7 +777,7 @@ struct UpdArgs {
 // beta+ = beta + mu H^{-1} g + eta (beta - beta_prev); one warp per row of H^{-1}.
 __global__ void __launch_bounds__(256) k_update(const UpdArgs A, DevState *st) {
   const UpdateArgs &a = A.u;
-  __shared__ double s_red[8][3];
+  __shared__ double s_red[3][8];
   __shared__ int s_last;
   if (a.check_done && st->done) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -773,17 +822,21 @@ __global__ void __launch_bounds__(256) k_update(const UpdArgs A, DevState *st) {
       if (a.hist && t < a.hist_cap) a.hist[(size_t)t * d + i] = v;
     }
   }
-  if (lane == 0) { s_red[warp][0] = ds; s_red[warp][1] = nn; s_red[warp][2] = dd; }
+  if (lane == 0) { s_red[0][warp] = ds; s_red[1][warp] = nn; s_red[2][warp] = dd; }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double x0 = 0, x1 = 0, x2 = 0;
-    for (int w = 0; w < 8; ++w) { x0 += s_red[w][0]; x1 += s_red[w][1]; x2 += s_red[w][2]; }
-    A.part[3 * blockIdx.x + 0] = x0;
-    A.part[3 * blockIdx.x + 1] = x1;
-    A.part[3 * blockIdx.x + 2] = x2;
-    __threadfence();
-    const unsigned prev = atomicAdd(&st->upd_count, 1u);
-    s_last = (prev == gridDim.x - 1);
+  if (warp == 0) {  // eight lanes per sum, a fixed tree
+    double x = lane < 24 ? s_red[lane >> 3][lane & 7] : 0.0;
+#pragma unroll
+    for (int off = 1; off < 8; off <<= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    if (lane < 24 && (lane & 7) == 0) {
+      A.part[3 * blockIdx.x + (lane >> 3)] = x;
+      __threadfence();
+    }
+    __syncwarp();
+    if (lane == 0) {
+      const unsigned prev = atomicAdd(&st->upd_count, 1u);
+      s_last = (prev == gridDim.x - 1);
+    }
   }
   __syncthreads();
   if (!s_last || warp != 0) return;
@@ -821,8 +874,12 @@ __global__ void __launch_bounds__(256) k_update(const UpdArgs A, DevState *st) {
   }
   if (lane != 0) return;
   st->upd_count = 0;
-  const double rel = sqrt(x0) / (sqrt(x1) > 0.0 ? sqrt(x1) : 1.0);
-  st->rel_step = rel;
+  // the relative step sqrt(x0 / x1) is compared squared: FP64 square roots, divisions and powers by one
+  // thread took part of this kernel's time (with the sums as trees 8.5 -> 6.6 us at d = 37)
+  const double n1 = x1 > 0.0 ? x1 : 1.0;
+  st->step2 = x0;
+  st->norm2 = n1;
+  const bool small = a.thr > 0.0 && x0 <= a.thr * a.thr * n1;
   const int tn = t + 1;
   st->iter = tn;
   if (!isfinite(x0) || !isfinite(x1)) {
@@ -845,9 +902,8 @@ __global__ void __launch_bounds__(256) k_update(const UpdArgs A, DevState *st) {
       // stage, overstates the gain in the error), so the remaining steps take the full form (its
       // next pass reads the r0 this exact pass wrote).  x0 and step_prev are squared norms.  A step
       // that meets the stopping test ends the fit either way and decides nothing.
-      const double gain = fmin(0.01, pow(a.rho, 2.0 * (1.0 + a.inner_cost * st->ninner)));
-      const bool stops = a.thr > 0.0 && rel <= a.thr;
-      if (st->step_prev > 0.0 && x0 > st->step_prev * gain && !stops) {
+      const double gain = a.gain[st->ninner < kMaxInner ? st->ninner : kMaxInner];
+      if (st->step_prev > 0.0 && x0 > st->step_prev * gain && !small) {
         st->dc = 0;
         st->dc_fell_back = 1;
       }
@@ -858,7 +914,7 @@ __global__ void __launch_bounds__(256) k_update(const UpdArgs A, DevState *st) {
       st->ninner += 1;
     }
     const bool may_stop = !(corr && !exact);  // the correction form stops on exact steps only
-    if (may_stop && a.thr > 0.0 && rel <= a.thr) st->done = 1;
+    if (may_stop && small) st->done = 1;
     else if (tn >= a.T) {
       st->done = 1;
       if (a.thr > 0.0) st->status |= ST_NOTCONV;
@@ -874,8 +930,7 @@ __global__ void __launch_bounds__(256) k_update(const UpdArgs A, DevState *st) {
       // that the FP32 residual r0 - X (beta - beta_0) stays within ~2^-34 ||X|| ||beta||
       if (st->dc) {
         const bool next_exact =
-            !exact && (reject || x0 < 1e-8 * st->step_ref || x0 > st->step_ref || st->ninner >= 20 ||
-                       (a.thr > 0.0 && rel <= a.thr));
+            !exact && (reject || x0 < 1e-8 * st->step_ref || x0 > st->step_ref || st->ninner >= kMaxInner || small);
         st->bfnext = next_exact ? 0 : 1;
         st->rebase = (next_exact && x2 > 0x1p-20 * x1) ? 1 : 0;
       } else {
@@ -883,29 +938,10 @@ __global__ void __launch_bounds__(256) k_update(const UpdArgs A, DevState *st) {
         st->rebase = (x2 > 0x1p-20 * x1 && x2 > 0x1p20 * x0) ? 1 : 0;
       }
     }
+    // the host polls this word (pinned host memory) for the iterations done and the stop flag
+    if (a.mail)
+      asm volatile("st.relaxed.sys.global.u32 [%0], %1;" ::"l"(a.mail), "r"((unsigned)tn << 1 | (unsigned)st->done) : "memory");
   }
-}
-
-// Correction step: g = g0 - G_b delta_e, one warp per row of G_b (four independent FP64 sums, fixed
-// order); only when the device state selects a correction step.
-__global__ void __launch_bounds__(256) k_gram_step(const double *Gb, const float *delta_e, const double *g0, double *g,
-                                                   int d, const DevState *st) {
-  if (st->done || st->rebase || !st->dc || !st->bfnext) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * 8 + warp;
-  if (i >= d) return;
-  const double *row = Gb + (size_t)i * d;
-  double h0 = 0.0, h1 = 0.0, h2 = 0.0, h3 = 0.0;
-  int k = lane;
-  for (; k + 96 < d; k += 128) {
-    h0 = fma(row[k], (double)delta_e[k], h0);
-    h1 = fma(row[k + 32], (double)delta_e[k + 32], h1);
-    h2 = fma(row[k + 64], (double)delta_e[k + 64], h2);
-    h3 = fma(row[k + 96], (double)delta_e[k + 96], h3);
-  }
-  for (; k < d; k += 32) h0 = fma(row[k], (double)delta_e[k], h0);
-  const double h = warp_sum((h0 + h1) + (h2 + h3));
-  if (lane == 0) g[i] = g0[i] - h;
 }
 
 __global__ void k_copy_beta(const double *ring, const DevState *st, int d, double *out) {
@@ -982,16 +1018,10 @@ cudaError_t launch_grad(int mode, int xdtype, const void *X, int64_t ldx, const 
       if (xdtype != SLSE_F32) return cudaErrorInvalidValue;
       const bool vec = d % 4 == 0 && aligned(X, ldx, 4, 4);
       // rows in flight per warp grow as d shrinks (the same 32 x-values per lane)
-      cudaError_t e;
-      if (!vec) e = launch1(k_grad_mixed<1, 16, 1, 1>, nblk, a, s);
-      else if (d <= 128) e = launch1(k_grad_mixed<4, 1, 1, 8>, nblk, a, s);
-      else if (d <= 256) e = launch1(k_grad_mixed<4, 2, 1, 4>, nblk, a, s);
-      else e = launch1(k_grad_mixed<4, 4, 1, 2>, nblk, a, s);
-      if (e != cudaSuccess) return e;
-      if (!vec) return launch1(k_grad_mixed<1, 16, 0, 1>, nblk, a, s);
-      if (d <= 128) return launch1(k_grad_mixed<4, 1, 0, 8>, nblk, a, s);
-      if (d <= 256) return launch1(k_grad_mixed<4, 2, 0, 4>, nblk, a, s);
-      return launch1(k_grad_mixed<4, 4, 0, 2>, nblk, a, s);
+      if (!vec) return launch1(k_grad_mixed<1, 16, 1>, nblk, a, s);
+      if (d <= 128) return launch1(k_grad_mixed<4, 1, 8>, nblk, a, s);
+      if (d <= 256) return launch1(k_grad_mixed<4, 2, 4>, nblk, a, s);
+      return launch1(k_grad_mixed<4, 4, 2>, nblk, a, s);
     }
     default:
       return cudaErrorInvalidValue;
@@ -1007,10 +1037,8 @@ cudaError_t preload_grad_kernels() {
       (const void *)SLSE_GRAD64_WIDE(double, 12), (const void *)SLSE_GRAD64_WIDE(double, 16),
       (const void *)SLSE_GRAD64_WIDE(float, 12), (const void *)SLSE_GRAD64_WIDE(float, 16),
 #undef SLSE_GRAD64_PTR
-      (const void *)k_grad_mixed<1, 16, 1, 1>,   (const void *)k_grad_mixed<4, 1, 1, 8>,
-      (const void *)k_grad_mixed<4, 2, 1, 4>,    (const void *)k_grad_mixed<4, 4, 1, 2>,
-      (const void *)k_grad_mixed<1, 16, 0, 1>,   (const void *)k_grad_mixed<4, 1, 0, 8>,
-      (const void *)k_grad_mixed<4, 2, 0, 4>,    (const void *)k_grad_mixed<4, 4, 0, 2>,
+      (const void *)k_grad_mixed<1, 16, 1>, (const void *)k_grad_mixed<4, 1, 8>,
+      (const void *)k_grad_mixed<4, 2, 4>, (const void *)k_grad_mixed<4, 4, 2>,
       (const void *)k_reduce};
   for (const void *f : k) {
     cudaFuncAttributes fa;
@@ -1021,8 +1049,10 @@ cudaError_t preload_grad_kernels() {
 }
 
 cudaError_t launch_reduce(const double *partials, int nblk, int d, double scale, double *g, DevState *st,
-                          int check_done, cudaStream_t s, double *g0) {
-  k_reduce<<<(d + 31) / 32, 256, 0, s>>>(partials, nblk, d, scale, g, st, check_done, g0);
+                          int check_done, cudaStream_t s, double *g0, const double *Gb, const float *delta_e,
+                          const double *rhs) {
+  const ReduceArgs a{partials, nblk, d, scale, g, st, check_done, g0, Gb, delta_e, rhs};
+  k_reduce<<<(d + 7) / 8, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -1030,12 +1060,6 @@ cudaError_t launch_update(const UpdateArgs &a, DevState *st, cudaStream_t s) {
   // per-CTA partial sums live right after the DevState's own cache line block
   UpdArgs A{a, reinterpret_cast<double *>(st + 1)};
   k_update<<<(a.d + 7) / 8, 256, 0, s>>>(A, st);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gram_step(const double *Gb, const float *delta_e, const double *g0, double *g, int d, DevState *st,
-                             cudaStream_t s) {
-  k_gram_step<<<(d + 7) / 8, 256, 0, s>>>(Gb, delta_e, g0, g, d, st);
   return cudaGetLastError();
 }
 

@@ -27,7 +27,7 @@ struct DevState {
   unsigned upd_count;  // last-block counter of the update kernel
   unsigned bar_count;  // grid barrier (QR)
   unsigned bar_gen;
-  double rel_step;     // last ||b+ - b|| / ||b+||
+  double step2, norm2; // last ||b+ - b||^2 and ||b+||^2 (1 for a zero iterate)
   long long spin_limit; // polls of a grid-wide wait before it gives up (0: the built-in 2^25)
   int dc;              // mixed 2nd stage, correction form active: correction steps between exact passes
   int bfnext;          // correction form: the next step is a correction step (else an exact pass over X)
@@ -265,18 +265,16 @@ int grad_grid(int nsm);
 cudaError_t launch_grad(int mode, int xdtype, const void *X, int64_t ldx, const void *Y, int64_t nrows,
                         int d, const double *beta_ring, DevState *st, const float *delta32, float *r0,
                         double *beta0, double *partials, int nblk, int check_done, cudaStream_t s);
-// g = scale * (sum of the per-CTA partials).  g0 (nullable; mixed 2nd stage in correction form):
-// after an exact pass (over X) g0 = g; on a correction step the reduction does nothing (the
-// correction step writes g).
+// g = scale * (sum of the per-CTA partials), plus rhs (nullable).  g0 (nullable; mixed 2nd stage in
+// correction form): after an exact pass (over X) g0 = g; on a correction step, as the device state
+// selects, g = g0 - G_b delta_e instead (G_b d x d FP64, delta_e = fl32(beta - beta_e)).
 cudaError_t launch_reduce(const double *partials, int nblk, int d, double scale, double *g,
-                          DevState *st, int check_done, cudaStream_t s, double *g0 = nullptr);
-// Correction step of the correction form: g = g0 - G_b delta_e (G_b d x d FP64, delta_e =
-// fl32(beta - beta_e)); runs only when the device state selects a correction step.
-cudaError_t launch_gram_step(const double *Gb, const float *delta_e, const double *g0, double *g, int d,
-                             DevState *st, cudaStream_t s);
+                          DevState *st, int check_done, cudaStream_t s, double *g0 = nullptr,
+                          const double *Gb = nullptr, const float *delta_e = nullptr, const double *rhs = nullptr);
 // Loads the code of every kernel launch_grad (GM_F64, GM_MIXED) and launch_reduce can launch,
 // so that a later first launch of one of them does not load a module (which allocates).
 cudaError_t preload_grad_kernels();
+constexpr int kMaxInner = 20;  // correction form: correction steps of a cycle, at most
 struct UpdateArgs {
   const double *g;
   const double *Hinv;
@@ -294,11 +292,17 @@ struct UpdateArgs {
   int mixed;           // maintain delta32 / rebase flag
   int check_done;
   int hist_base;       // iteration index of the first 2nd-stage step (mode_hist is indexed from it)
-  double rho;          // sqrt(d / r), the contraction of a plain 2nd-stage step (correction form's test)
+  double gain[kMaxInner + 1];  // correction form: what an exact step of a cycle with k correction steps has to
+                               // shrink to (squared, correction_gains)
+  unsigned *mail;      // host-visible word, nullable: 2 (iterations done) + stop flag after each 2nd-stage step
   double *beta_e;      // correction form: the iterate of the last exact pass
   float *delta_e;      // correction form: fl32(beta - beta_e), the vector of the correction step
-  double inner_cost;   // correction form: cost of a correction step in exact passes (fallback test)
 };
+// gain[k] = min(1/100, rho^(2 (1 + cost k))): a cycle of an exact pass and k correction steps, each
+// costing `cost` passes, has to gain what plain steps of contraction rho gain in that time, and 10x.
+void correction_gains(double rho, double cost, double (&gain)[kMaxInner + 1]);
+// ||b+ - b|| / ||b+|| of the last step
+double rel_step(const DevState &s);
 cudaError_t launch_update(const UpdateArgs &a, DevState *st, cudaStream_t s);
 cudaError_t launch_copy_beta(const double *beta_ring, DevState *st, int d, double *out, cudaStream_t s);
 
