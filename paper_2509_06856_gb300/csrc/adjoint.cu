@@ -256,8 +256,12 @@ struct AdjLayout {
   size_t o_g0, o_be, o_de, o_gb, o_gram, total;
 };
 
-// From this many elements of X on the backward solve takes the correction form (off).
-constexpr int64_t kAdjCorrection = INT64_MAX;
+// From this many elements of X on the backward solve takes the correction form: a pass then costs more
+// than a correction step and the solve's ~25 passes more than the Gram build (one to three of them).
+// Below, a pass is a few microseconds of launch latency like the step.  Measured, full against
+// correction form (us): 2^16 x 128 808, 847; 2^17 x 128 927, 862; 2^18 x 128 1372, 942; 2^18 x 512
+// 2831, 1651; 2^20 x 512 8108, 3217; 2^21 x 32 4838, 1752.
+constexpr int64_t kAdjCorrection = int64_t(1) << 24;
 
 AdjLayout adj_layout(const slse_problem *p, int prec, int nsm) {
   AdjLayout L{};
