@@ -18,7 +18,7 @@ LIB = os.path.join(PKG, "libslse.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I" + os.path.join(ROOT, "include")]
-SOURCES = ["api.cu", "draws.cu", "srht.cu", "srht64.cu", "srht_tc.cu", "grad.cu", "linalg.cu", "noalloc.cu", "countsketch.cu", "adjoint.cu", "fp8.cu",
+SOURCES = ["api.cu", "draws.cu", "srht.cu", "srht64.cu", "srht_tc.cu", "grad.cu", "linalg.cu", "qr.cu", "noalloc.cu", "countsketch.cu", "adjoint.cu", "fp8.cu",
            "gaussian.cu", "gram.cu"]
 
 

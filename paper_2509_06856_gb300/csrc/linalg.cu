@@ -424,7 +424,8 @@ int qr_grid(int64_t r, int nsm) {
 
 size_t qr_ws_bytes(int64_t r, int d, int nsm) {
   const int G = qr_grid(r, nsm);
-  return align256(2 * (size_t)G * d * 8) + 2 * align256(2 * (size_t)d * 8) + 2 * align256((size_t)d * d * 8);
+  return align256(2 * (size_t)G * d * 8) + 2 * align256(2 * (size_t)d * 8) + 2 * align256((size_t)d * d * 8) +
+         (qr_panels_ok(r) ? align256(qr_panels_ws_bytes(r, d)) : 0);
 }
 
 cudaError_t launch_gather_hessian_rows(int prec, const void *U, int64_t ldu, int64_t row0, int64_t r, int d,
@@ -447,19 +448,6 @@ cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, doubl
   e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const int G = qr_grid(r, nsm);
-  const int64_t nr_max = (r + G - 1) / G;
-  const size_t smem = (size_t)nr_max * d * sizeof(double);
-  const bool use_smem = smem <= (size_t)200 * 1024;
-  auto kern = use_smem ? k_qr<true> : k_qr<false>;
-  const size_t dyn = use_smem ? smem : 0;
-  if (use_smem) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e != cudaSuccess) return e;
-  }
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kQrThreads, dyn);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
   char *p = static_cast<char *>(ws);
   size_t off = 0;
   QrArgs a;
@@ -474,9 +462,28 @@ cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, doubl
   double *Rinv = reinterpret_cast<double *>(p + off); off += align256((size_t)d * d * 8);
   a.Rt = reinterpret_cast<double *>(p + off); off += align256((size_t)d * d * 8);
   a.st = st;
-  void *args[] = {&a};
-  e = cudaLaunchCooperativeKernel((const void *)kern, dim3(G), dim3(kQrThreads), args, dyn, s);
-  if (e != cudaSuccess) return e;
+  // by panels up to 16384 rows (their rows stay in a cluster's registers); the column-by-column form
+  // above that, and when a test limits the polls of its grid barrier (the panels have no such wait)
+  if (qr_panels_ok(r) && debug_spin_limit() == 0) {
+    if ((e = launch_qr_panels(A, r, d, lda, R, a.Rt, p + off, st, s)) != cudaSuccess) return e;
+  } else {
+    const int64_t nr_max = (r + G - 1) / G;
+    const size_t smem = (size_t)nr_max * d * sizeof(double);
+    const bool use_smem = smem <= (size_t)200 * 1024;
+    auto kern = use_smem ? k_qr<true> : k_qr<false>;
+    const size_t dyn = use_smem ? smem : 0;
+    if (use_smem) {
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+      if (e != cudaSuccess) return e;
+    }
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kQrThreads, dyn);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    void *args[] = {&a};
+    e = cudaLaunchCooperativeKernel((const void *)kern, dim3(G), dim3(kQrThreads), args, dyn, s);
+    if (e != cudaSuccess) return e;
+  }
   if (Hinv) {
     k_tri_inv_sweep<<<(d + 7) / 8, 256, 0, s>>>(R, a.Rt, d, Rinv, st);
     const int nt = (d + 31) / 32;

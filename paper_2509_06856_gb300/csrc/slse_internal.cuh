@@ -306,6 +306,13 @@ double rel_step(const DevState &s);
 cudaError_t launch_update(const UpdateArgs &a, DevState *st, cudaStream_t s);
 cudaError_t launch_copy_beta(const double *beta_ring, DevState *st, int d, double *out, cudaStream_t s);
 
+// qr.cu: Householder QR by panels.  R (non-negative diagonal) and R^T of the r x d matrix A (row-major,
+// not modified); r within qr_panels_ok.  An exactly zero column raises ST_NUMERIC.
+bool qr_panels_ok(int64_t r);
+size_t qr_panels_ws_bytes(int64_t r, int d);
+cudaError_t launch_qr_panels(const double *A, int64_t r, int d, int64_t lda, double *R, double *Rt, void *ws, DevState *st,
+                             cudaStream_t s);
+
 // linalg.cu
 size_t qr_ws_bytes(int64_t r, int d, int nsm);
 cudaError_t launch_gather_hessian_rows(int prec, const void *U, int64_t ldu, int64_t row0, int64_t r,
