@@ -145,8 +145,9 @@ typedef struct {
                              stream (overlaps ms_draws): Y, and X unless the first SRHT pass reads it */
   double ms_draws, ms_sketch, ms_qr, ms_stage1, ms_stage2, ms_total; /* CUDA-event phase times */
   double ms_srht_pass1, ms_srht_pass2; /* the two sketch passes (pass 2 is 0 for single-pass sizes) */
-  double ms_grad2;        /* summed CUDA-event time of the 2nd-stage gradient launches */
-  int32_t n_grad2;        /* number of those launches that did a full pass */
+  double ms_grad2;        /* summed device-clock time of the 2nd-stage passes over X, each from the end of the
+                             step before to the end of the pass */
+  int32_t n_grad2;        /* number of those passes */
   int32_t kernels;        /* kernel launches made by the call */
   int32_t iters_stage1, iters_stage2;
   double final_rel_step;  /* ||b_T - b_{T-1}|| / ||b_T|| of the last iteration */
@@ -154,8 +155,8 @@ typedef struct {
   double bytes_grad2;     /* algorithmic HBM bytes of one 2nd-stage gradient pass */
   int32_t rebases;        /* mixed path: number of 2nd-stage residual re-bases (exact passes) */
   int32_t status;
-  double ms_corr;         /* SLSE_STAGE2_CORRECTION: summed CUDA-event time of the correction steps (not
-                             included in ms_grad2, which then covers the exact passes over X) */
+  double ms_corr;         /* SLSE_STAGE2_CORRECTION: summed device-clock time of the correction steps' products
+                             (not included in ms_grad2, which then covers the exact passes over X) */
   int32_t n_corr;         /* number of correction steps */
   int32_t stage2_full;    /* 1 if a correction run fell back to the full form */
   double ms_gram;         /* CUDA-event time of forming the Gram matrix of the BF16 rounding of X */

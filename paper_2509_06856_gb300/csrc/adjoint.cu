@@ -404,12 +404,12 @@ extern "C" slse_status slse_solve_normal(const slse_problem *prob, const double 
   ua.mail = const_cast<unsigned *>(word);
   for (int k = 0; k < sched->T; ++k) {
     if (launch_grad(mixed ? GM_MIXED : GM_F64, prob->dtype, prob->X, prob->ldx, y0, prob->N, d, ring, st, d32, r0, b0,
-                    part, L.nblk, 1, s) != cudaSuccess)
+                    part, L.nblk, 1, s, true) != cudaSuccess)
       return SLSE_ECUDA;
     // v + X^T (0 - X w), or the correction step's product
-    if (launch_reduce(part, L.nblk, d, 1.0, g, st, 1, s, g0, Gb, de, v) != cudaSuccess) return SLSE_ECUDA;
+    if (launch_reduce(part, L.nblk, d, 1.0, g, st, 1, s, g0, Gb, de, v, true) != cudaSuccess) return SLSE_ECUDA;
     ua.first = k == 0;
-    if (launch_update(ua, st, s) != cudaSuccess) return SLSE_ECUDA;
+    if (launch_update(ua, st, s, true) != cudaSuccess) return SLSE_ECUDA;
     launches += 3;
     // iteration k+1 is enqueued before iteration k is awaited
     if (k > 0) {

@@ -320,6 +320,9 @@ __global__ void k_set_stage2(DevState *st, int rebase, int dc) {
     st->step_ref = 0.0;
     st->step_prev = 0.0;
     st->ninner = 0;
+    st->ns_pass = 0;
+    st->ns_corr = 0;
+    st->t_mark = device_ns();
   }
 }
 
@@ -669,6 +672,11 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
   ua.hist = tr ? tr->beta_hist : nullptr; ua.hist_cap = hist_cap; ua.d = d; ua.mu = s.mu; ua.eta = s.eta;
   ua.T = T;
 
+  // The iteration's kernels are dependent launches (their CTAs wait in place), except beside a long Gram
+  // build: the waiting CTAs take the gaps in which its CTAs get onto the SMs.  Measured: mixed fit of
+  // 100003 x 37 1.32 -> 1.04 ms, FP64 fit of 20000 x 50 1.42 -> 1.25, CountSketch fit of 1500001 x 256
+  // 3.81 -> 3.70; 2^22 x 512 13.4 -> 14.0 ms with them beside the build (from 2 to 4.8 ms long).
+  const bool dep_early = !L.dc || (double)p->N * d < 0x1p29;
   // a8 stage 1: a_i M-IHS steps on each nested sketch (prefix of the sampled rows)
   int t = 0;
   for (size_t i = 0; i < s.m.size() && t < T; ++i) {
@@ -681,14 +689,14 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
     for (int j = 0; j < s.a[i] && t < T; ++j) {
       if (fp8)
         CK(launch_grad_mx(static_cast<const uint8_t *>(Ui), L.ldu, Us + r0w * L.nsb, L.nsb,
-                          static_cast<const __nv_bfloat16 *>(Vi), m, d, ring, dst, part, nb, st));
+                          static_cast<const __nv_bfloat16 *>(Vi), m, d, ring, dst, part, nb, st, dep_early));
       else
         CK(launch_grad(mixed ? GM_STAGE1_BF16 : GM_STAGE1_F64, mixed ? SLSE_BF16 : SLSE_F64, Ui, L.ldu, Vi, m, d,
-                       ring, dst, nullptr, nullptr, nullptr, part, nb, 0, st));
-      CK(launch_reduce(part, nb, d, sq_scale(m), g, dst, 0, st));
+                       ring, dst, nullptr, nullptr, nullptr, part, nb, 0, st, dep_early));
+      CK(launch_reduce(part, nb, d, sq_scale(m), g, dst, 0, st, nullptr, nullptr, nullptr, nullptr, dep_early));
       ua.first = (j == 0 && s.momentum_reset) || t == 0;
       ua.stage2 = 0; ua.thr = 0.0; ua.mixed = 0; ua.check_done = 0;
-      CK(launch_update(ua, dst, st));
+      CK(launch_update(ua, dst, st, dep_early));
       kernels += 3;
       CK(mark_iter(t));
       ++t;
@@ -702,7 +710,6 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
   // stop flag is already set.  The update kernel writes iterations and flag to pinned host memory,
   // which the host polls: a copy and an event per step, two more events created and five launches
   // made this loop host-bound (small fits 44 -> 29 us a step).
-  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> e_grad;
   // correction form: the Gram matrix G_b of the BF16 copy of X (formed once, here), g(beta_e)
   // beside the gradient, the iterate beta_e of the last exact pass and fl32(beta - beta_e)
   double *g0 = L.dc ? reinterpret_cast<double *>(base + L.o_g0) : nullptr;
@@ -738,21 +745,16 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
     *word = (unsigned)t << 1;
     ua.mail = const_cast<unsigned *>(word);
     for (int k = 0; t + k < T; ++k) {
-      cudaEvent_t g0e = E.make(), g1 = E.make();
-      if (!g0e || !g1) return SLSE_ECUDA;
       if (k == 1) CK(join_gram());
-      CK(cudaEventRecord(g0e, st));
+      const bool dep = dep_early || k > 0;
       // correction form: a pass over X (exact) or a correction step g = g(beta_e) - G_b (beta - beta_e),
       // as the device state selects (the pass returns at once on a correction step)
       CK(launch_grad(mixed ? GM_MIXED : GM_F64, p->dtype, p->X, p->ldx, p->Y, p->N, d, ring, dst, d32, r0, b0,
-                     part, nb, 1, st));
-      if (!L.dc) CK(cudaEventRecord(g1, st));
-      CK(launch_reduce(part, nb, d, 1.0, g, dst, 1, st, g0, Gb, de));  // or the correction step's product
-      if (L.dc) CK(cudaEventRecord(g1, st));
-      e_grad.emplace_back(g0e, g1);
+                     part, nb, 1, st, dep));
+      CK(launch_reduce(part, nb, d, 1.0, g, dst, 1, st, g0, Gb, de, nullptr, dep));
       ua.first = (k == 0 && s.momentum_reset) || (t + k) == 0;
       ua.stage2 = 1; ua.thr = thr; ua.mixed = mixed ? 1 : 0; ua.check_done = 1;
-      CK(launch_update(ua, dst, st));
+      CK(launch_update(ua, dst, st, dep));
       kernels += 3;
       CK(mark_iter(t + k));
       if (k > 0) {
@@ -794,25 +796,14 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
     RP->ms_stage1 = ms_between(e_qr, e_s1);
     RP->ms_total = ms_between(e_start, e_end);
     RP->ms_stage2 = RP->ms_total - ms_between(e_start, e_s1);
-    // gradient launches that ran a full pass (the speculative one after the stop returns at once),
-    // split by pass kind: over X (exact or full form) or over its BF16 copy (correction form)
+    // passes over X (exact or full form) and correction steps, by the device clock
     const int full = fin.iter - t1;
-    double mg = 0.0, mb16 = 0.0;
-    int nx = 0, nb16 = 0;
-    for (int k = 0; k < full && k < (int)e_grad.size(); ++k) {
-      const double ms = ms_between(e_grad[k].first, e_grad[k].second);
-      if (k < (int)sizeof(fin.mode_hist) && fin.mode_hist[k] == 1) {
-        mb16 += ms;
-        ++nb16;
-      } else {
-        mg += ms;
-        ++nx;
-      }
-    }
-    RP->ms_grad2 = mg;
+    int nx = 0, nc = 0;
+    for (int k = 0; k < full; ++k) (k < (int)sizeof(fin.mode_hist) && fin.mode_hist[k] == 1 ? nc : nx) += 1;
+    RP->ms_grad2 = 1e-6 * (double)fin.ns_pass;
     RP->n_grad2 = nx;
-    RP->ms_corr = mb16;
-    RP->n_corr = nb16;
+    RP->ms_corr = 1e-6 * (double)fin.ns_corr;
+    RP->n_corr = nc;
     RP->stage2_full = fin.dc_fell_back;
     if (L.dc && e_gram0) {
       RP->ms_gram = ms_between(e_gram0, e_gram1);

@@ -43,6 +43,7 @@ template <int RPW>
 __global__ void __launch_bounds__(kThreads, 2) k_grad_mx(const uint8_t *U, int64_t ldq, const uint8_t *S, int64_t nsb,
                                                          const __nv_bfloat16 *V, int64_t nrows, int d,
                                                          const double *beta_ring, const DevState *st, double *part) {
+  dependent_start();
   __shared__ double sm[kWarps][512];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = (int64_t)blockIdx.x * kWarps + warp, nw = (int64_t)gridDim.x * kWarps;
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_grad_mx(const uint8_t *U, int64
 __global__ void __launch_bounds__(kThreads) k_grad_mx_s(const uint8_t *U, int64_t ldq, const uint8_t *S, int64_t nsb,
                                                         const __nv_bfloat16 *V, int64_t nrows, int d,
                                                         const double *beta_ring, const DevState *st, double *part) {
+  dependent_start();
   __shared__ double sm[kWarps][512];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = (int64_t)blockIdx.x * kWarps + warp, nw = (int64_t)gridDim.x * kWarps;
@@ -185,12 +187,11 @@ unsigned grid_for(int64_t n, int threads) {
 
 cudaError_t launch_grad_mx(const uint8_t *U, int64_t ldq, const uint8_t *S, int64_t nsb, const __nv_bfloat16 *V,
                            int64_t nrows, int d, const double *beta_ring, const DevState *st, double *part, int nblk,
-                           cudaStream_t s) {
+                           cudaStream_t s, bool dep) {
   if (d < 1 || d > 512) return cudaErrorInvalidValue;
   const bool vec = d % 16 == 0 && ldq % 16 == 0 && reinterpret_cast<uintptr_t>(U) % 16 == 0;
-  if (vec) k_grad_mx<4><<<nblk, kThreads, 0, s>>>(U, ldq, S, nsb, V, nrows, d, beta_ring, st, part);
-  else k_grad_mx_s<<<nblk, kThreads, 0, s>>>(U, ldq, S, nsb, V, nrows, d, beta_ring, st, part);
-  return cudaGetLastError();
+  return launch_dep(vec ? k_grad_mx<4> : k_grad_mx_s, (unsigned)nblk, kThreads, 0, s, dep, U, ldq, S, nsb, V, nrows, d,
+                    beta_ring, st, part);
 }
 
 cudaError_t launch_mx_to_bf16(const uint8_t *U, int64_t ldq, const uint8_t *S, int64_t nsb, int64_t rows, int d,

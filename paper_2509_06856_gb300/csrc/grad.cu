@@ -209,6 +209,7 @@ template <class Tx, int VW, int VMAX, int RPW, bool BS>
 __global__ void __launch_bounds__(kGradThreads, 2) k_grad_f64(const GradArgs a) {
   extern __shared__ __align__(16) unsigned char ring_raw[];
   __shared__ __align__(16) double sm[kWarps][512];
+  dependent_start();
   if (a.check_done && a.st->done) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = (int64_t)blockIdx.x * kWarps + warp, nw = (int64_t)gridDim.x * kWarps;
@@ -407,6 +408,7 @@ __device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 
 template <int VMAX, int RPW>
 __global__ void __launch_bounds__(kGradThreads, 2) k_grad_bf16v(const GradArgs a) {
   __shared__ double sm[kWarps][512];
+  dependent_start();
   if (a.check_done && a.st->done) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = (int64_t)blockIdx.x * kWarps + warp, nw = (int64_t)gridDim.x * kWarps;
@@ -486,6 +488,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_grad_bf16v(const GradArgs a
 template <int VMAX>
 __global__ void __launch_bounds__(kGradThreads) k_grad_bf16s(const GradArgs a) {
   __shared__ double sm[kWarps][512];
+  dependent_start();
   if (a.check_done && a.st->done) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = (int64_t)blockIdx.x * kWarps + warp, nw = (int64_t)gridDim.x * kWarps;
@@ -776,6 +779,7 @@ __device__ __forceinline__ void grad_mixed_body(const GradArgs &a, double (*sm)[
 template <int VW, int VMAX, int RPW>
 __global__ void __launch_bounds__(kGradThreads, 2) k_grad_mixed(const GradArgs a) {
   __shared__ __align__(16) double sm[kWarps][512];
+  dependent_start();
   if (a.check_done && a.st->done) return;
   if (a.st->rebase) {
     grad_mixed_body<VW, VMAX, 1, RPW>(a, sm);
@@ -791,7 +795,7 @@ struct ReduceArgs {
   int nblk, d;
   double scale;
   double *g;
-  const DevState *st;
+  DevState *st;
   int check_done;
   double *g0;            // correction form: g(beta_e)
   const double *Gb;      // correction form: the Gram matrix and fl32(beta - beta_e)
@@ -806,7 +810,9 @@ struct ReduceArgs {
 // four chains; the correction step's product used to be a launch of its own (2.6 us).
 __global__ void __launch_bounds__(256) k_reduce(const ReduceArgs a) {
   __shared__ double sm[8][8];
-  const DevState *st = a.st;
+  dependent_start();
+  DevState *st = a.st;
+  if (blockIdx.x == 0 && threadIdx.x == 0) st->t_red = device_ns();
   if (a.check_done && st->done) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, d = a.d;
   if (a.g0 && st->dc && st->bfnext && !st->rebase) {
@@ -866,7 +872,9 @@ __global__ void __launch_bounds__(256) k_update(const UpdArgs A, DevState *st) {
   const UpdateArgs &a = A.u;
   __shared__ double s_red[3][8];
   __shared__ int s_last;
+  dependent_start();
   if (a.check_done && st->done) return;
+  if (a.stage2 && blockIdx.x == 0 && threadIdx.x == 0) st->t_upd = device_ns();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int d = a.d;
   const int t = st->iter;
@@ -979,6 +987,9 @@ __global__ void __launch_bounds__(256) k_update(const UpdArgs A, DevState *st) {
     const int exact = !corr || st->rebase || !st->bfnext;  // this iteration's pass was over X
     const int k2 = t - a.hist_base;
     if (k2 >= 0 && k2 < (int)sizeof(st->mode_hist)) st->mode_hist[k2] = exact ? 0 : 1;
+    if (exact) st->ns_pass += st->t_red - st->t_mark;
+    else st->ns_corr += st->t_upd - st->t_mark;
+    st->t_mark = device_ns();
     if (corr && exact) {
       // a cycle (exact pass + k correction steps, 1 + k c passes' worth of time for a correction
       // step costing c passes) that shrank the exact step by less than rho^(1 + k c), what plain
@@ -1037,9 +1048,8 @@ __global__ void k_copy_beta(const double *ring, const DevState *st, int d, doubl
 }
 
 template <class K>
-cudaError_t launch1(K kern, int nblk, const GradArgs &a, cudaStream_t s) {
-  kern<<<nblk, kGradThreads, 0, s>>>(a);
-  return cudaGetLastError();
+cudaError_t launch1(K kern, int nblk, const GradArgs &a, cudaStream_t s, bool dep) {
+  return launch_dep(kern, (unsigned)nblk, kGradThreads, 0, s, dep, a);
 }
 
 // FP64 kernel with its register tile sized to d (columns per lane) and several rows per warp
@@ -1052,14 +1062,13 @@ cudaError_t launch1(K kern, int nblk, const GradArgs &a, cudaStream_t s) {
   F(8, (VW == 1 ? 2 : 1), (k_grad_f64<Tx, VW, 8, (VW == 1 ? 2 : 1), (VW == 2)>))
 #define SLSE_GRAD64_WIDE(Tx, V) (k_grad_f64<Tx, 1, V, 1, true>)
 template <class Tx, int VW>
-cudaError_t launch_f64(int d, int nblk, const GradArgs &a, cudaStream_t s) {
+cudaError_t launch_f64(int d, int nblk, const GradArgs &a, cudaStream_t s, bool dep) {
   constexpr int per = 32 * VW;
   auto go = [&](auto kern, size_t row_bytes, int rows) -> cudaError_t {
     const size_t smem = (size_t)kWarps * 2 * rows * row_bytes;  // at most 64 KB
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<nblk, kGradThreads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_dep(kern, (unsigned)nblk, kGradThreads, smem, s, dep, a);
   };
 #define SLSE_GRAD64_CASE(V, R, K) if (d <= V * per) return go(K, V * per * sizeof(Tx), R);
   SLSE_GRAD64_VARIANTS(Tx, VW, SLSE_GRAD64_CASE)
@@ -1081,37 +1090,36 @@ int grad_grid(int nsm) { return 2 * nsm; }
 
 cudaError_t launch_grad(int mode, int xdtype, const void *X, int64_t ldx, const void *Y, int64_t nrows, int d,
                         const double *beta_ring, DevState *st, const float *delta32, float *r0, double *beta0,
-                        double *partials, int nblk, int check_done, cudaStream_t s) {
+                        double *partials, int nblk, int check_done, cudaStream_t s, bool dep) {
   GradArgs a{X, ldx, Y, nrows, d, beta_ring, st, delta32, r0, beta0, partials, check_done};
   if (d > 512 || d < 1) return cudaErrorInvalidValue;
   switch (mode) {
     case GM_F64:
     case GM_STAGE1_F64:
       if (xdtype == SLSE_F64) {
-        if (d % 2 == 0 && aligned(X, ldx, 8, 2)) return launch_f64<double, 2>(d, nblk, a, s);
-        return launch_f64<double, 1>(d, nblk, a, s);
+        if (d % 2 == 0 && aligned(X, ldx, 8, 2)) return launch_f64<double, 2>(d, nblk, a, s, dep);
+        return launch_f64<double, 1>(d, nblk, a, s, dep);
       } else {
-        if (d % 2 == 0 && aligned(X, ldx, 4, 2)) return launch_f64<float, 2>(d, nblk, a, s);
-        return launch_f64<float, 1>(d, nblk, a, s);
+        if (d % 2 == 0 && aligned(X, ldx, 4, 2)) return launch_f64<float, 2>(d, nblk, a, s, dep);
+        return launch_f64<float, 1>(d, nblk, a, s, dep);
       }
     case GM_STAGE1_BF16:
       // the sketch buffer's padding columns are never written: the vector path requires
       // d % 8 == 0 so that no padding word is read
       // lanes cover 8 columns per word: one word per lane up to d = 256 (more rows in flight)
       if (d % 8 == 0 && ldx % 8 == 0 && aligned(X, ldx, 2, 8))
-        return d <= 256 ? launch1(k_grad_bf16v<1, 6>, nblk, a, s) : launch1(k_grad_bf16v<2, 4>, nblk, a, s);
-      return launch1(k_grad_bf16s<16>, nblk, a, s);
+        return d <= 256 ? launch1(k_grad_bf16v<1, 6>, nblk, a, s, dep) : launch1(k_grad_bf16v<2, 4>, nblk, a, s, dep);
+      return launch1(k_grad_bf16s<16>, nblk, a, s, dep);
     case GM_MIXED: {
       if (xdtype != SLSE_F32) return cudaErrorInvalidValue;
       const bool vec = d % 4 == 0 && aligned(X, ldx, 4, 4);
       // rows in flight per warp grow as d shrinks (the same 32 x-values per lane)
-      if (!vec) return launch1(k_grad_mixed<1, 16, 1>, nblk, a, s);
+      if (!vec) return launch1(k_grad_mixed<1, 16, 1>, nblk, a, s, dep);
       auto go = [&](auto kern) -> cudaError_t {
         constexpr int smem = kWarps * 2 * 8 * 32 * 16;  // two stages of eight 16-byte pieces per lane
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        kern<<<nblk, kGradThreads, smem, s>>>(a);
-        return cudaGetLastError();
+        return launch_dep(kern, (unsigned)nblk, kGradThreads, smem, s, dep, a);
       };
       if (d <= 128) return go(k_grad_mixed<4, 1, 8>);
       if (d <= 256) return go(k_grad_mixed<4, 2, 4>);
@@ -1144,17 +1152,15 @@ cudaError_t preload_grad_kernels() {
 
 cudaError_t launch_reduce(const double *partials, int nblk, int d, double scale, double *g, DevState *st,
                           int check_done, cudaStream_t s, double *g0, const double *Gb, const float *delta_e,
-                          const double *rhs) {
+                          const double *rhs, bool dep) {
   const ReduceArgs a{partials, nblk, d, scale, g, st, check_done, g0, Gb, delta_e, rhs};
-  k_reduce<<<(d + 7) / 8, 256, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_dep(k_reduce, (unsigned)(d + 7) / 8, 256, 0, s, dep, a);
 }
 
-cudaError_t launch_update(const UpdateArgs &a, DevState *st, cudaStream_t s) {
+cudaError_t launch_update(const UpdateArgs &a, DevState *st, cudaStream_t s, bool dep) {
   // per-CTA partial sums live right after the DevState's own cache line block
   UpdArgs A{a, reinterpret_cast<double *>(st + 1)};
-  k_update<<<(a.d + 7) / 8, 256, 0, s>>>(A, st);
-  return cudaGetLastError();
+  return launch_dep(k_update, (unsigned)(a.d + 7) / 8, 256, 0, s, dep, A, st);
 }
 
 cudaError_t launch_copy_beta(const double *beta_ring, DevState *st, int d, double *out, cudaStream_t s) {

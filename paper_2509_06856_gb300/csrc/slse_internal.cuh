@@ -35,9 +35,42 @@ struct DevState {
   double step_ref;     // correction form: squared step of the last exact pass
   double step_prev;    // correction form: squared step of the exact pass before it
   int ninner;          // correction form: correction steps since the last exact pass
+  // device clock (ns): end of the last 2nd-stage step, start of this step's reduction and update, and the
+  // time of the passes over X and of the correction steps' products so far
+  unsigned long long t_mark, t_red, t_upd, ns_pass, ns_corr;
   unsigned char mode_hist[128];  // 2nd-stage step kind of iteration t (< 128): 0 pass over X, 1 correction step
 };
 static_assert(sizeof(DevState) <= 512, "the per-CTA partials of the update kernel follow the state");
+
+// ----------------------------------------------------------------------------------
+// Programmatic dependent launch of the iteration's kernels: each lets its successor's CTAs be placed
+// while it runs and itself starts with the wait for its predecessor (complete, its writes visible), so
+// a launch costs no gap.  Without the launch attribute both instructions do nothing.
+__device__ __forceinline__ void dependent_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ unsigned long long device_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+// kern<<<grid, block, smem, s>>>(args...), as a dependent launch when `dep`
+template <class... P, class... A>
+inline cudaError_t launch_dep(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, bool dep,
+                              A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = dep ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 // ----------------------------------------------------------------------------------
 // Philox4x32-10 (Salmon et al., SC'11).  Counter (c0..c3), key (k0, k1).
@@ -156,7 +189,7 @@ cudaError_t launch_countsketch(const CsPlan &pl, int xdtype, const void *X, int6
 // block of a row, byte = exponent + 127; Y values in BF16).
 cudaError_t launch_grad_mx(const uint8_t *U, int64_t ldq, const uint8_t *S, int64_t nsb, const __nv_bfloat16 *V,
                            int64_t nrows, int d, const double *beta_ring, const DevState *st, double *part, int nblk,
-                           cudaStream_t s);
+                           cudaStream_t s, bool dep = false);
 cudaError_t launch_mx_to_bf16(const uint8_t *U, int64_t ldq, const uint8_t *S, int64_t nsb, int64_t rows, int d,
                               __nv_bfloat16 *out, int64_t ldo, cudaStream_t s);
 cudaError_t launch_quantize_mx(const __nv_bfloat16 *A, int64_t lda, int64_t rows, int d, uint8_t *U, int64_t ldq,
@@ -264,13 +297,14 @@ enum GradMode { GM_F64 = 0, GM_MIXED = 1, GM_STAGE1_BF16 = 2, GM_STAGE1_F64 = 3 
 int grad_grid(int nsm);
 cudaError_t launch_grad(int mode, int xdtype, const void *X, int64_t ldx, const void *Y, int64_t nrows,
                         int d, const double *beta_ring, DevState *st, const float *delta32, float *r0,
-                        double *beta0, double *partials, int nblk, int check_done, cudaStream_t s);
+                        double *beta0, double *partials, int nblk, int check_done, cudaStream_t s, bool dep = false);
 // g = scale * (sum of the per-CTA partials), plus rhs (nullable).  g0 (nullable; mixed 2nd stage in
 // correction form): after an exact pass (over X) g0 = g; on a correction step, as the device state
 // selects, g = g0 - G_b delta_e instead (G_b d x d FP64, delta_e = fl32(beta - beta_e)).
 cudaError_t launch_reduce(const double *partials, int nblk, int d, double scale, double *g,
                           DevState *st, int check_done, cudaStream_t s, double *g0 = nullptr,
-                          const double *Gb = nullptr, const float *delta_e = nullptr, const double *rhs = nullptr);
+                          const double *Gb = nullptr, const float *delta_e = nullptr, const double *rhs = nullptr,
+                          bool dep = false);
 // Loads the code of every kernel launch_grad (GM_F64, GM_MIXED) and launch_reduce can launch,
 // so that a later first launch of one of them does not load a module (which allocates).
 cudaError_t preload_grad_kernels();
@@ -303,7 +337,7 @@ struct UpdateArgs {
 void correction_gains(double rho, double cost, double (&gain)[kMaxInner + 1]);
 // ||b+ - b|| / ||b+|| of the last step
 double rel_step(const DevState &s);
-cudaError_t launch_update(const UpdateArgs &a, DevState *st, cudaStream_t s);
+cudaError_t launch_update(const UpdateArgs &a, DevState *st, cudaStream_t s, bool dep = false);
 cudaError_t launch_copy_beta(const double *beta_ring, DevState *st, int d, double *out, cudaStream_t s);
 
 // qr.cu: Householder QR by panels.  R (non-negative diagonal) and R^T of the r x d matrix A (row-major,
