@@ -11,7 +11,7 @@
 // operand of tcgen05.mma (8 x 16-byte core matrices); k_gauss_tc gives each CTA 128 rows of
 // G and a range of chunks, in a pipeline of up to 8 stages.  Sixteen producer warps draw the
 // G tile in FP32 (hardware log2, sin, cos, rsqrt; the Philox words of the next chunk are drawn
-// beside the Box-Muller step of the current one), round it to BF16 and store it in the same
+// beside the Box-Muller step of the current one; four groups of warps draw a chunk each), round it to BF16 and store it in the same
 // layout; one thread copies the X chunk with cp.async.bulk; one thread issues the
 // 128 x ncp x 32 MMAs into an FP32 accumulator in tensor memory; four warps read it back
 // (tcgen05.ld) into per-split partial sums, which k_gauss_reduce adds in a fixed order.
@@ -116,11 +116,15 @@ constexpr int kBM = 128;               // rows of G per CTA (MMA M)
 constexpr int kBK = 32;                // rows of X per chunk
 constexpr int kSBO = kBK * 16;         // bytes between 8-row groups of a tile
 constexpr int kTileA = kBM * kBK * 2;  // 8 KiB
-constexpr int kProdWarps = 16;         // 512 producer threads: one Philox call (8 entries) each per chunk
+constexpr int kProdWarps = 16;
+// Groups of producer warps, each drawing whole chunks: a thread then waits, fences and arrives once per
+// kGroups Philox calls, and one group's waiting is another's drawing.  Measured (GB300), 3072 rows of G,
+// 524288 x 512, the whole call: 1.86 ms with the 16 warps on one chunk, 1.78 with 2 groups, 1.68 with 4.
+constexpr int kGroups = 4;
 constexpr int kLoadWarp = kProdWarps, kMmaWarp = kProdWarps + 1;
 constexpr int kTcThreads = (kProdWarps + 2) * 32;
 constexpr int kMaxStages = 8;
-static_assert(kProdWarps * 32 == kBM * (kBK / 8), "one 8-entry octet per producer thread and chunk");
+static_assert(kProdWarps * 32 == kBM * (kBK / 8), "a group's threads have kGroups 8-entry octets each per chunk");
 
 struct TcArgs {
   const uint8_t *xt;   // nchunk packed X chunks of ncp * 64 bytes
@@ -154,7 +158,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gauss_tc(const TcArgs a) {
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
-      mbar_init(&full_g[s], kProdWarps);  // one arrival per producer warp
+      mbar_init(&full_g[s], kProdWarps / kGroups);  // one arrival per producer warp of a group
       mbar_init(&full_x[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -178,35 +182,49 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gauss_tc(const TcArgs a) {
   const int64_t m0 = (int64_t)blockIdx.x * kBM;
 
   if (warp < kProdWarps) {
-    // producers: row = thread mod 128, octet (8 entries along K) = thread div 128
-    const int row = threadIdx.x & (kBM - 1);
-    const int oct = threadIdx.x >> 7;
+    // producers: group grp draws the whole tiles of chunks grp, grp + kGroups, ...; thread tg of a
+    // group has row tg mod 128 and octets (8 entries along K) tg div 128 + j (4 / kGroups)
+    constexpr int kOctStep = (kBK / 8) / kGroups;
+    const int grp = warp / (kProdWarps / kGroups);
+    const int tg = threadIdx.x - grp * (kProdWarps / kGroups * 32);
+    const int row = tg & (kBM - 1);
+    const int oct = tg >> 7;
     const int64_t gi = m0 + row;
     const bool live = gi < a.m;
     uint8_t *dst0 = sA + (row >> 3) * kSBO + (row & 7) * 16 + oct * 128;
-    // the Philox words of chunk k + 1 are drawn beside the Box-Muller step of chunk k (two
-    // independent dependency chains per thread)
+    // the Philox words of the group's next chunk are drawn beside the Box-Muller step of this one
     const RoundKeys K = round_keys(a.seed_lo, a.seed_hi);
-    uint64_t q = (uint64_t)c0 * (kBK / 8) + (uint64_t)oct;  // octet index of chunk k along K
-    U4 wn = philox_rk((uint32_t)q, (uint32_t)(q >> 32), kStreamG, (uint32_t)gi, K);
-    int s = 0;
+    uint64_t q = (uint64_t)(c0 + grp) * (kBK / 8) + (uint64_t)oct;  // octet index along K
+    auto words = [&](int j) {
+      const uint64_t qj = q + (uint64_t)(j * kOctStep);
+      return philox_rk((uint32_t)qj, (uint32_t)(qj >> 32), kStreamG, (uint32_t)gi, K);
+    };
+    U4 wn[kGroups];
+#pragma unroll
+    for (int j = 0; j < kGroups; ++j) wn[j] = words(j);
+    int s = grp;
     uint32_t ph = 0;
-    for (int k = 0; k < nk; ++k) {
+    for (int k = grp; k < nk; k += kGroups) {
+      uint4 v[kGroups];
+      if (k + kGroups < nk) q += kGroups * (kBK / 8);
+#pragma unroll
+      for (int j = 0; j < kGroups; ++j) {
+        const U4 w = wn[j];
+        wn[j] = words(j);
+        const uint2 v01 = box_muller_bf16x2_pair(w.x, w.y), v23 = box_muller_bf16x2_pair(w.z, w.w);
+        v[j] = live ? make_uint4(v01.x, v01.y, v23.x, v23.y) : make_uint4(0u, 0u, 0u, 0u);
+      }
       // warp-uniform: a lane that gave up takes its whole warp out of the loop
       if (!__all_sync(0xFFFFFFFFu, mbar_wait(&empty[s], ph ^ 1u, abort_f, a.status))) break;
-      const U4 w = wn;
-      if (k + 1 < nk) q += kBK / 8;
-      wn = philox_rk((uint32_t)q, (uint32_t)(q >> 32), kStreamG, (uint32_t)gi, K);
-      const uint2 v01 = box_muller_bf16x2_pair(w.x, w.y), v23 = box_muller_bf16x2_pair(w.z, w.w);
-      uint4 v = make_uint4(v01.x, v01.y, v23.x, v23.y);
-      if (!live) v = make_uint4(0u, 0u, 0u, 0u);
-      *reinterpret_cast<uint4 *>(dst0 + (size_t)s * kTileA) = v;
-      // each thread orders its own store before the MMA's (async-proxy) read; the warp then
+#pragma unroll
+      for (int j = 0; j < kGroups; ++j)
+        *reinterpret_cast<uint4 *>(dst0 + (size_t)s * kTileA + j * kOctStep * 128) = v[j];
+      // each thread orders its own stores before the MMA's (async-proxy) read; the warp then
       // arrives once
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&full_g[s]);
-      if (++s == S) { s = 0; ph ^= 1u; }
+      if ((s += kGroups) >= S) { s -= S; ph ^= 1u; }
     }
     if (warp < 4) {
       // epilogue: TMEM lanes 32 warp .. 32 warp + 31 hold rows m0 + 32 warp + lane
