@@ -159,7 +159,7 @@ struct FitLayout {
   GramWPlan gwp;
   size_t o_gpart;           // its partial sums, inside the big region after W and its Y column
   size_t o_xin, o_yin, o_g0, o_be, o_de, o_gb, o_gst;
-  size_t o_state, o_psd, o_sigma, o_pos, o_big, o_wy, o_u, o_v, o_A, o_R, o_Hinv, o_qr, o_chol, o_part, o_g,
+  size_t o_state, o_psd, o_sigma, o_pos, o_big, o_wy, o_u, o_v, o_A, o_R, o_Hinv, o_qr, o_qrp, total_min, o_chol, o_part, o_g,
       o_ring, o_b0, o_d32, o_out, o_r0, o_us, o_hat16;
   size_t total;
 };
@@ -253,6 +253,9 @@ FitLayout fit_layout(const slse_problem *p, const Sched &s, int nsm) {
     L.o_xin = w.take((size_t)p->N * d * bx);
     L.o_yin = w.take((size_t)p->N * bx);
   }
+  // the panels' copy of A comes last: a fit given a workspace without it factors column by column
+  L.total_min = w.total;
+  L.o_qrp = w.take(s.prec == SLSE_PREC_FP64 && qr_panels_ok(s.r) ? qr_panels_ws_bytes(s.r, d) : 0);
   L.total = w.total;
   return L;
 }
@@ -406,7 +409,8 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
   const FitLayout L = fit_layout(pin, s, nsm);
   if (is_host_pointer(pin->Y) != L.host_in) return SLSE_EINVAL;  // X and Y in the same kind of memory
   Workspace W;
-  slse_status a = acquire(W, ws_user, ws_bytes, L.total, st);
+  const bool panels = L.total > L.total_min && (!ws_user || ws_bytes >= L.total);
+  slse_status a = acquire(W, ws_user, ws_bytes, panels ? L.total : L.total_min, st);
   if (a != SLSE_OK) return a;
   char *base = static_cast<char *>(W.ptr);
   slse_problem prob = *pin;  // device view of the inputs
@@ -657,7 +661,7 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
                                     std::sqrt(hat_scale2), A, st));
       ++kernels;
     }
-    CK(launch_qr(A, s.r, d, d, R, Hinv, qrws, dst, st));
+    CK(launch_qr(A, s.r, d, d, R, Hinv, qrws, panels ? base + L.o_qrp : nullptr, dst, st));
     kernels += 3;
   }
   CK(cudaEventRecord(e_qr, st));
@@ -894,6 +898,7 @@ size_t slse_workspace_size(const slse_problem *prob, const slse_schedule *sched,
       w.take(kStateBytes);
       w.take((size_t)arg * prob->d * 8);
       w.take(qr_ws_bytes(arg, prob->d, nsm));
+      if (qr_panels_ok(arg)) w.take(qr_panels_ws_bytes(arg, prob->d));
       return w.total;
     }
     default:
@@ -1062,8 +1067,12 @@ slse_status slse_qr(const double *A, int64_t r, int32_t d, int64_t lda, double *
   const size_t o_state = w.take(kStateBytes);
   const size_t o_a = w.take((size_t)r * d * 8);
   const size_t o_qr = w.take(qr_ws_bytes(r, d, nsm));
+  // a workspace without room for the panels' copy factors column by column
+  const size_t total_min = w.total;
+  const size_t o_qrp = w.take(qr_panels_ok(r) ? qr_panels_ws_bytes(r, d) : 0);
+  const bool panels = w.total > total_min && (!workspace || ws_bytes >= w.total);
   Workspace W;
-  slse_status a = acquire(W, workspace, ws_bytes, w.total, st);
+  slse_status a = acquire(W, workspace, ws_bytes, panels ? w.total : total_min, st);
   if (a != SLSE_OK) return a;
   char *base = static_cast<char *>(W.ptr);
   DevState *dst = reinterpret_cast<DevState *>(base + o_state);
@@ -1071,7 +1080,7 @@ slse_status slse_qr(const double *A, int64_t r, int32_t d, int64_t lda, double *
   k_init_state<<<1, 32, 0, st>>>(dst, 0, debug_spin_limit());
   CK(cudaGetLastError());
   CK(cudaMemcpy2DAsync(Ac, (size_t)d * 8, A, (size_t)lda * 8, (size_t)d * 8, (size_t)r, cudaMemcpyDeviceToDevice, st));
-  CK(launch_qr(Ac, r, d, d, R, Hinv, base + o_qr, dst, st));
+  CK(launch_qr(Ac, r, d, d, R, Hinv, base + o_qr, panels ? base + o_qrp : nullptr, dst, st));
   return SLSE_OK;
 }
 

@@ -424,8 +424,7 @@ int qr_grid(int64_t r, int nsm) {
 
 size_t qr_ws_bytes(int64_t r, int d, int nsm) {
   const int G = qr_grid(r, nsm);
-  return align256(2 * (size_t)G * d * 8) + 2 * align256(2 * (size_t)d * 8) + 2 * align256((size_t)d * d * 8) +
-         (qr_panels_ok(r) ? align256(qr_panels_ws_bytes(r, d)) : 0);
+  return align256(2 * (size_t)G * d * 8) + 2 * align256(2 * (size_t)d * 8) + 2 * align256((size_t)d * d * 8);
 }
 
 cudaError_t launch_gather_hessian_rows(int prec, const void *U, int64_t ldu, int64_t row0, int64_t r, int d,
@@ -439,9 +438,10 @@ cudaError_t launch_gather_hessian_rows(int prec, const void *U, int64_t ldu, int
   return cudaGetLastError();
 }
 
-// A is overwritten (it must be a scratch copy).  ws: qr_ws_bytes(r, d).
-cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, double *Hinv, void *ws, DevState *st,
-                      cudaStream_t s) {
+// A is overwritten (it must be a scratch copy).  ws: qr_ws_bytes(r, d); panels: qr_panels_ws_bytes(r, d)
+// or nullptr (column by column).
+cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, double *Hinv, void *ws, void *panels,
+                      DevState *st, cudaStream_t s) {
   int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -464,8 +464,8 @@ cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, doubl
   a.st = st;
   // by panels up to 16384 rows (their rows stay in a cluster's registers); the column-by-column form
   // above that, and when a test limits the polls of its grid barrier (the panels have no such wait)
-  if (qr_panels_ok(r) && debug_spin_limit() == 0) {
-    if ((e = launch_qr_panels(A, r, d, lda, R, a.Rt, p + off, st, s)) != cudaSuccess) return e;
+  if (panels && qr_panels_ok(r) && debug_spin_limit() == 0) {
+    if ((e = launch_qr_panels(A, r, d, lda, R, a.Rt, panels, st, s)) != cudaSuccess) return e;
   } else {
     const int64_t nr_max = (r + G - 1) / G;
     const size_t smem = (size_t)nr_max * d * sizeof(double);

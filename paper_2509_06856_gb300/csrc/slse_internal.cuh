@@ -351,7 +351,7 @@ cudaError_t launch_qr_panels(const double *A, int64_t r, int d, int64_t lda, dou
 size_t qr_ws_bytes(int64_t r, int d, int nsm);
 cudaError_t launch_gather_hessian_rows(int prec, const void *U, int64_t ldu, int64_t row0, int64_t r,
                                        int d, double scale, double *A, cudaStream_t s);
-cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, double *Hinv, void *ws,
+cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, double *Hinv, void *ws, void *panels,
                       DevState *st, cudaStream_t s);
 // Mixed path: H-hat^{-1} = G^{-1} for G = scale2 * U[row0:row0+r]^T U[row0:row0+r] (U in BF16,
 // G accumulated exactly), by the blocked sweep operator in FP64.  A non-positive pivot

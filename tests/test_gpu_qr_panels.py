@@ -37,3 +37,21 @@ def test_zero_column_raises_enumeric():
     sched = slse.default_schedule(4096, 24, T=20, tol=1e-10)
     res = slse.fit(dev(X), dev(X[:, 0].copy()), sched, seed=2, raise_on_error=False)
     assert res.status == slse.ENUMERIC
+
+
+def test_fit_with_a_workspace_without_the_panels_scratch():
+    """One 256-byte unit less than the full workspace: the factor column by column, the same fit within
+    the error of either factor; a workspace short by far more stays refused."""
+    torch = torch_cuda()
+    import paper_2509_06856_gb300 as slse
+    rng = np.random.default_rng(4)
+    N, d = 5000, 40
+    X = rng.standard_normal((N, d))
+    Xd, Yd = dev(X), dev(X @ rng.standard_normal(d) + 0.1 * rng.standard_normal(N))
+    sched = slse.default_schedule(N, d, prec="fp64", T=60, tol=1e-13)
+    full = slse.workspace_size(Xd, Yd, slse.OP_FIT, sched)
+    b = [slse.fit(Xd, Yd, sched, seed=6, workspace=slse.alloc_workspace(n)).beta for n in (full, full - 256)]
+    # both stop at the fixed point of the same FP64 iteration (tol 1e-13, condition below 2)
+    assert np.linalg.norm(b[0] - b[1]) <= 1e-11 * np.linalg.norm(b[0])
+    with pytest.raises(slse.SlseError):
+        slse.fit(Xd, Yd, sched, seed=6, workspace=slse.alloc_workspace(full // 2))
