@@ -636,10 +636,16 @@ cudaError_t launch_pass_t(const GroupArgs &a, int L, int64_t ngroups, cudaStream
     case 7: e = launch_group_t<Tin, Ts, Tout, 7, 1, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s); break;
     case 8: e = launch_group_t<Tin, Ts, Tout, 8, 1, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s); break;
     case 9: e = launch_group_t<Tin, Ts, Tout, 8, 2, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s); break;
-    case 10: e = launch_group_t<Tin, Ts, Tout, 8, 4, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s); break;
-    case 11: e = launch_group_t<Tin, Ts, Tout, 8, 8, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s); break;
     case 12: e = launch_group_t<Tin, Ts, Tout, 9, 8, CP, VA, VB, VO, 3, 4, CPY>(a, ngroups, s); break;
-    default: return cudaErrorInvalidValue;
+    default:
+      // W is always aligned: a BF16 pass 2 of these groups never gets here
+      if constexpr (std::is_same_v<Tin, __nv_bfloat16> && std::is_same_v<Tout, __nv_bfloat16>) {
+        return cudaErrorInvalidValue;
+      } else {
+        if (L != 10 && L != 11) return cudaErrorInvalidValue;
+        e = L == 10 ? launch_group_t<Tin, Ts, Tout, 8, 4, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s)
+                    : launch_group_t<Tin, Ts, Tout, 8, 8, CP, VA, VB, VO, MB, 4, CPY>(a, ngroups, s);
+      }
   }
   if (e != cudaSuccess) return e;
   const size_t ysm = (size_t)(1 << L) * sizeof(Ts);
