@@ -9,9 +9,9 @@
 //
 // MIXED_BF16 (X F32): X is packed once into BF16 chunks of 32 rows laid out as the K-major
 // operand of tcgen05.mma (8 x 16-byte core matrices); k_gauss_tc gives each CTA 128 rows of
-// G and a range of chunks, in a pipeline of up to 8 stages.  Sixteen producer warps draw the
+// G and a range of chunks, in a pipeline of up to 8 stages.  The producer warps draw the
 // G tile in FP32 (hardware log2, sin, cos, rsqrt; the Philox words of the next chunk are drawn
-// beside the Box-Muller step of the current one; four groups of warps draw a chunk each), round it to BF16 and store it in the same
+// beside the Box-Muller step of the current one; each group of four warps draws a chunk), round it to BF16 and store it in the same
 // layout; one thread copies the X chunk with cp.async.bulk; one thread issues the
 // 128 x ncp x 32 MMAs into an FP32 accumulator in tensor memory; four warps read it back
 // (tcgen05.ld) into per-split partial sums, which k_gauss_reduce adds in a fixed order.
@@ -116,15 +116,19 @@ constexpr int kBM = 128;               // rows of G per CTA (MMA M)
 constexpr int kBK = 32;                // rows of X per chunk
 constexpr int kSBO = kBK * 16;         // bytes between 8-row groups of a tile
 constexpr int kTileA = kBM * kBK * 2;  // 8 KiB
-constexpr int kProdWarps = 16;
-// Groups of producer warps, each drawing whole chunks: a thread then waits, fences and arrives once per
-// kGroups Philox calls, and one group's waiting is another's drawing.  Measured (GB300), 3072 rows of G,
-// 524288 x 512, the whole call: 1.86 ms with the 16 warps on one chunk, 1.78 with 2 groups, 1.68 with 4.
-constexpr int kGroups = 4;
-constexpr int kLoadWarp = kProdWarps, kMmaWarp = kProdWarps + 1;
-constexpr int kTcThreads = (kProdWarps + 2) * 32;
+// Groups of four producer warps, each drawing whole chunks: a thread then waits, fences and arrives once
+// per four Philox calls, and one group's waiting is another's drawing.  Measured (GB300), 6 d rows of G, the
+// whole call: 524288 x 512 1.86 ms with 16 warps on one chunk, 1.78 with 2 groups, 1.68 with 4;
+// up to 256 packed columns, where the ring has eight stages, five groups (2^20 x 256 1.71 -> 1.63 ms,
+// 524288 x 200 0.73 -> 0.70); at 512 columns, with five stages, five groups lose (1.73 -> 1.80).  The draws
+// bound the kernel: 1.65 ms for 524288 x 512 without the MMAs, 1.25 without the draws, 1.71 without the
+// copies of X.  More G stages beside the X stages let the groups fall into step and lost (1.91 ms), as
+// did X chunks shared by a pair of CTAs (1.89).
+constexpr int kGroupWarps = 4;  // a thread per row of the tile
+constexpr int kOct = kBK / 8;   // octets (8 entries along K) of a thread in a chunk: one Philox call each
+constexpr int tc_threads(int groups) { return (groups * kGroupWarps + 2) * 32; }
 constexpr int kMaxStages = 8;
-static_assert(kProdWarps * 32 == kBM * (kBK / 8), "a group's threads have kGroups 8-entry octets each per chunk");
+static_assert(kGroupWarps * 32 == kBM, "one row per thread of a group");
 
 struct TcArgs {
   const uint8_t *xt;   // nchunk packed X chunks of ncp * 64 bytes
@@ -141,7 +145,9 @@ struct TcArgs {
 // Pipeline per CTA (rows m0 .. m0 + 127 of G, chunks c0 .. c1 - 1): stage s of S holds one G
 // tile (producer warps) and one X chunk (bulk copy); the MMA thread waits for both, issues the
 // chunk's MMAs and commits them to empty[s], which frees the stage for both producers.
-__global__ void __launch_bounds__(kTcThreads, 1) k_gauss_tc(const TcArgs a) {
+template <int kGroups>
+__global__ void __launch_bounds__(tc_threads(kGroups), 1) k_gauss_tc(const TcArgs a) {
+  constexpr int kProdWarps = kGroups * kGroupWarps, kLoadWarp = kProdWarps, kMmaWarp = kProdWarps + 1;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int S = a.stages;
@@ -158,7 +164,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gauss_tc(const TcArgs a) {
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
-      mbar_init(&full_g[s], kProdWarps / kGroups);  // one arrival per producer warp of a group
+      mbar_init(&full_g[s], kGroupWarps);  // one arrival per producer warp of a group
       mbar_init(&full_x[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -182,33 +188,29 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gauss_tc(const TcArgs a) {
   const int64_t m0 = (int64_t)blockIdx.x * kBM;
 
   if (warp < kProdWarps) {
-    // producers: group grp draws the whole tiles of chunks grp, grp + kGroups, ...; thread tg of a
-    // group has row tg mod 128 and octets (8 entries along K) tg div 128 + j (4 / kGroups)
-    constexpr int kOctStep = (kBK / 8) / kGroups;
-    const int grp = warp / (kProdWarps / kGroups);
-    const int tg = threadIdx.x - grp * (kProdWarps / kGroups * 32);
-    const int row = tg & (kBM - 1);
-    const int oct = tg >> 7;
+    // producers: group grp draws the whole tiles of chunks grp, grp + kGroups, ...; one row per thread
+    const int grp = warp / kGroupWarps;
+    const int row = threadIdx.x - grp * kBM;
     const int64_t gi = m0 + row;
     const bool live = gi < a.m;
-    uint8_t *dst0 = sA + (row >> 3) * kSBO + (row & 7) * 16 + oct * 128;
+    uint8_t *dst0 = sA + (row >> 3) * kSBO + (row & 7) * 16;
     // the Philox words of the group's next chunk are drawn beside the Box-Muller step of this one
     const RoundKeys K = round_keys(a.seed_lo, a.seed_hi);
-    uint64_t q = (uint64_t)(c0 + grp) * (kBK / 8) + (uint64_t)oct;  // octet index along K
+    uint64_t q = (uint64_t)(c0 + grp) * kOct;  // octet index along K
     auto words = [&](int j) {
-      const uint64_t qj = q + (uint64_t)(j * kOctStep);
+      const uint64_t qj = q + (uint64_t)j;
       return philox_rk((uint32_t)qj, (uint32_t)(qj >> 32), kStreamG, (uint32_t)gi, K);
     };
-    U4 wn[kGroups];
+    U4 wn[kOct];
 #pragma unroll
-    for (int j = 0; j < kGroups; ++j) wn[j] = words(j);
+    for (int j = 0; j < kOct; ++j) wn[j] = words(j);
     int s = grp;
     uint32_t ph = 0;
     for (int k = grp; k < nk; k += kGroups) {
-      uint4 v[kGroups];
-      if (k + kGroups < nk) q += kGroups * (kBK / 8);
+      uint4 v[kOct];
+      if (k + kGroups < nk) q += kGroups * kOct;
 #pragma unroll
-      for (int j = 0; j < kGroups; ++j) {
+      for (int j = 0; j < kOct; ++j) {
         const U4 w = wn[j];
         wn[j] = words(j);
         const uint2 v01 = box_muller_bf16x2_pair(w.x, w.y), v23 = box_muller_bf16x2_pair(w.z, w.w);
@@ -217,8 +219,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gauss_tc(const TcArgs a) {
       // warp-uniform: a lane that gave up takes its whole warp out of the loop
       if (!__all_sync(0xFFFFFFFFu, mbar_wait(&empty[s], ph ^ 1u, abort_f, a.status))) break;
 #pragma unroll
-      for (int j = 0; j < kGroups; ++j)
-        *reinterpret_cast<uint4 *>(dst0 + (size_t)s * kTileA + j * kOctStep * 128) = v[j];
+      for (int j = 0; j < kOct; ++j)
+        *reinterpret_cast<uint4 *>(dst0 + (size_t)s * kTileA + j * 128) = v[j];
       // each thread orders its own stores before the MMA's (async-proxy) read; the warp then
       // arrives once
       fence_proxy_async_smem();
@@ -562,7 +564,9 @@ cudaError_t launch_gaussian(const GaussPlan &p, int xdtype, const void *X, int64
   if (xdtype != SLSE_F32) return cudaErrorInvalidValue;
   uint8_t *xt = base + p.o_xt;
   float *part = reinterpret_cast<float *>(base + p.o_part);
-  if ((e = cudaFuncSetAttribute(k_gauss_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem))) return e;
+  const bool five = p.ncp <= 256;
+  auto kern = five ? k_gauss_tc<5> : k_gauss_tc<4>;
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem))) return e;
   const int ncols = p.d + (p.with_y ? 1 : 0);
   for (int g = 0; g < p.groups; ++g) {
     const int c0 = 512 * g;
@@ -590,7 +594,7 @@ cudaError_t launch_gaussian(const GaussPlan &p, int xdtype, const void *X, int64
     a.tmem_cols = tc <= p.tmem_cols ? tc : p.tmem_cols;
     a.stages = p.stages;
     a.seed_lo = slo; a.seed_hi = shi;
-    k_gauss_tc<<<dim3((unsigned)(p.mpad / kBM), (unsigned)p.splits), kTcThreads, p.smem, s>>>(a);
+    kern<<<dim3((unsigned)(p.mpad / kBM), (unsigned)p.splits), tc_threads(five ? 5 : 4), p.smem, s>>>(a);
     if ((e = cudaGetLastError())) return e;
     const int64_t tot = p.m * ncp;
     const int rb = (int)(cdiv(tot, 256) < 8 * p.nsm ? cdiv(tot, 256) : 8 * p.nsm);
