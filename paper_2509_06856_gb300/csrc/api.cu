@@ -159,7 +159,7 @@ struct FitLayout {
   GramWPlan gwp;
   size_t o_gpart;           // its partial sums, inside the big region after W and its Y column
   size_t o_xin, o_yin, o_g0, o_be, o_de, o_gb, o_gst;
-  size_t o_state, o_psd, o_sigma, o_pos, o_big, o_wy, o_u, o_v, o_A, o_R, o_Hinv, o_qr, o_qrp, total_min, o_chol, o_part, o_g,
+  size_t o_state, o_psd, o_sigma, o_pos, o_big, o_wy, o_u, o_v, o_A, o_R, o_Hinv, o_qr, o_chol, o_part, o_g,
       o_ring, o_b0, o_d32, o_out, o_r0, o_us, o_hat16;
   size_t total;
 };
@@ -225,6 +225,9 @@ FitLayout fit_layout(const slse_problem *p, const Sched &s, int nsm) {
     L.grp = gram_plan(p->N, d, nsm);
     if (L.grp.total > big) big = L.grp.total;
   }
+  // FP64: the QR's panels copy A there, when the sketch's temporaries are dead too
+  if (s.prec == SLSE_PREC_FP64 && qr_panels_ok(s.r) && qr_panels_ws_bytes(s.r, d) > big)
+    big = qr_panels_ws_bytes(s.r, d);
   L.o_big = w.take(big);
   L.o_wy = L.o_big + align256(wbytes);
   L.o_u = w.take((size_t)L.n_samp * L.ldu * eu);
@@ -253,9 +256,6 @@ FitLayout fit_layout(const slse_problem *p, const Sched &s, int nsm) {
     L.o_xin = w.take((size_t)p->N * d * bx);
     L.o_yin = w.take((size_t)p->N * bx);
   }
-  // the panels' copy of A comes last: a fit given a workspace without it factors column by column
-  L.total_min = w.total;
-  L.o_qrp = w.take(s.prec == SLSE_PREC_FP64 && qr_panels_ok(s.r) ? qr_panels_ws_bytes(s.r, d) : 0);
   L.total = w.total;
   return L;
 }
@@ -409,8 +409,7 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
   const FitLayout L = fit_layout(pin, s, nsm);
   if (is_host_pointer(pin->Y) != L.host_in) return SLSE_EINVAL;  // X and Y in the same kind of memory
   Workspace W;
-  const bool panels = L.total > L.total_min && (!ws_user || ws_bytes >= L.total);
-  slse_status a = acquire(W, ws_user, ws_bytes, panels ? L.total : L.total_min, st);
+  slse_status a = acquire(W, ws_user, ws_bytes, L.total, st);
   if (a != SLSE_OK) return a;
   char *base = static_cast<char *>(W.ptr);
   slse_problem prob = *pin;  // device view of the inputs
@@ -661,7 +660,7 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
                                     std::sqrt(hat_scale2), A, st));
       ++kernels;
     }
-    CK(launch_qr(A, s.r, d, d, R, Hinv, qrws, panels ? base + L.o_qrp : nullptr, dst, st));
+    CK(launch_qr(A, s.r, d, d, R, Hinv, qrws, s.prec == SLSE_PREC_FP64 ? big : nullptr, dst, st));
     kernels += 3;
   }
   CK(cudaEventRecord(e_qr, st));

@@ -39,19 +39,23 @@ def test_zero_column_raises_enumeric():
     assert res.status == slse.ENUMERIC
 
 
-def test_fit_with_a_workspace_without_the_panels_scratch():
-    """One 256-byte unit less than the full workspace: the factor column by column, the same fit within
-    the error of either factor; a workspace short by far more stays refused."""
+def test_qr_with_a_workspace_without_the_panels_copy():
+    """One 256-byte unit less than the full workspace: the factor column by column, R within the error of
+    either factor (above); a workspace short by far more stays refused."""
     torch = torch_cuda()
     import paper_2509_06856_gb300 as slse
-    rng = np.random.default_rng(4)
-    N, d = 5000, 40
-    X = rng.standard_normal((N, d))
-    Xd, Yd = dev(X), dev(X @ rng.standard_normal(d) + 0.1 * rng.standard_normal(N))
-    sched = slse.default_schedule(N, d, prec="fp64", T=60, tol=1e-13)
-    full = slse.workspace_size(Xd, Yd, slse.OP_FIT, sched)
-    b = [slse.fit(Xd, Yd, sched, seed=6, workspace=slse.alloc_workspace(n)).beta for n in (full, full - 256)]
-    # both stop at the fixed point of the same FP64 iteration (tol 1e-13, condition below 2)
-    assert np.linalg.norm(b[0] - b[1]) <= 1e-11 * np.linalg.norm(b[0])
-    with pytest.raises(slse.SlseError):
-        slse.fit(Xd, Yd, sched, seed=6, workspace=slse.alloc_workspace(full // 2))
+    r, d = 700, 40
+    A = np.random.default_rng(4).standard_normal((r, d))
+    Ad = dev(A)
+    full = slse.workspace_size(Ad, Ad[:, 0].contiguous(), slse.OP_QR, arg=r)
+    got = []
+    for n in (full, full - 256, r * d * 4):
+        ws = slse.alloc_workspace(n)
+        R = torch.zeros((d, d), dtype=torch.float64, device="cuda")
+        st = slse._lib.slse_qr(Ad.data_ptr(), r, d, d, R.data_ptr(), None, ws.data_ptr(), n, slse._stream(None))
+        torch.cuda.synchronize()
+        got.append((st, host(R)))
+    assert [g[0] for g in got] == [slse.OK, slse.OK, slse.ENOMEM]
+    s = np.linalg.svd(A, compute_uv=False)
+    tol = 4 * np.sqrt(2) * s[0] / s[-1] * r * np.sqrt(d) * 2.0 ** -53 * np.linalg.norm(A)
+    assert np.linalg.norm(got[0][1] - got[1][1]) <= tol
