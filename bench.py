@@ -496,8 +496,8 @@ def run_ours(args, rank, ws, local_rank):
     ms_d, n_d, by_d = k_times[dom]
     achieved = by_d / (ms_d / n_d) / 1e6
     src = {"grad_stage2": ["paper_2509_06856_gb300/csrc/grad.cu"],
-           "srht_pass1": ["paper_2509_06856_gb300/csrc/srht.cu"],
-           "srht_pass2": ["paper_2509_06856_gb300/csrc/srht.cu"]}[dom]
+           "srht_pass1": ["paper_2509_06856_gb300/csrc/srht_tc.cu"],
+           "srht_pass2": ["paper_2509_06856_gb300/csrc/srht_tc.cu"]}[dom]
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": profile_traffic(dom, src), "kernel": dom, "peak_source": peak_kind,
                 "frac_of_nominal_8000": achieved / 8000.0}

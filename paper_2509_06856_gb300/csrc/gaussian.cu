@@ -11,8 +11,8 @@
 // operand of tcgen05.mma (8 x 16-byte core matrices); k_gauss_tc gives each CTA 128 rows of
 // G and a range of chunks, in a pipeline of up to 8 stages.  The producer warps draw the
 // G tile in FP32 (hardware log2, sin, cos, rsqrt; the Philox words of the next chunk are drawn
-// beside the Box-Muller step of the current one; each group of four warps draws a chunk), round it to BF16 and store it in the same
-// layout; one thread copies the X chunk with cp.async.bulk; one thread issues the
+// beside the Box-Muller step of the current one; each group of four warps draws a chunk), round it
+// to BF16 and store it in the same layout; one thread copies the X chunk with cp.async.bulk; one thread issues the
 // 128 x ncp x 32 MMAs into an FP32 accumulator in tensor memory; four warps read it back
 // (tcgen05.ld) into per-split partial sums, which k_gauss_reduce adds in a fixed order.
 // FP64: the same entries in double precision (log, sincospi) and an FP64 CUDA-core product.

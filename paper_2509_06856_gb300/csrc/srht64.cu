@@ -13,7 +13,7 @@
 // exchanges once through shared memory (three 32-bit planes) and takes the next five; sizes above
 // 2^10 take the remaining bits with warp shuffles.  No cluster: the exchange stays on the SM.
 //
-// Measured (GB300), sketch of 10^6 x 200 FP64 (N' = 2^20, 1/16 of the rows kept): 9.28 -> 3.30 ms
+// Measured (GB300), sketch of 10^6 x 200 FP64 (N' = 2^20, 1/16 of the rows kept): 9.27 -> 3.11 ms
 // against FP64 butterflies on clusters, error against 64-bit arithmetic 3.2e-16 -> 2.4e-16;
 // 2^20 x 256 11.3 -> 3.95 ms, 2^22 x 256 48.6 -> 18.1 ms, FP32 storage the same.  What bounds it
 // now: 118 warp instructions per element at 16 warps per SM, with the loads of a group exposed

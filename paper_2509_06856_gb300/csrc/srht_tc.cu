@@ -22,10 +22,10 @@
 // copies FP32 rows into three stages of its own (96 KB on their way), from which the same threads
 // split them into two operand stages.
 // Measured (GB300) against the cluster form: N' = 2^22, d = 512, FP32 in, half the rows kept: pass 1
-// 3.45 -> 3.00 ms, pass 2 3.22 -> 1.49 ms; sketch of 3000000 x 384 in BF16 5.38 -> 3.90 ms, its error
-// against 64-bit arithmetic unchanged (2.4e-3, the BF16 roundings).  What bounds pass 1 now: the
-// producers' splitting and the part of the epilogue that holds tensor memory (the loads alone would
-// take 2.2 ms).  Tried on the way: eight producer warps loading into registers (32 KB on their way
+// 3.45 -> 3.05 ms, pass 2 3.22 -> 1.49 ms; sketch of 3000000 x 384 in BF16 5.43 -> 3.65 ms (0.25 of it
+// by the draws' sort), its error against 64-bit arithmetic unchanged (2.4e-3, the BF16 roundings).  What bounds
+// pass 1 now: the producers' splitting and the part of the epilogue that holds tensor memory (the loads
+// alone would take 2.2 ms).  Tried on the way: eight producer warps loading into registers (32 KB on their way
 // per SM: 3.39 ms at 3000000 x 384, 2.24 ms now), eight epilogue warps, H as an MN-major operand (the MMAs ran at
 // half the rate), all output rows read back before the first store (spills).
 // Every mbarrier wait is bounded (ST_TIMEOUT); copies in flight are awaited and tensor memory is
