@@ -291,9 +291,8 @@ int32_t slse_default_schedule_for(int64_t N, int32_t d, int32_t kind, slse_sched
  * with the gradient v - X^T X w and the preconditioner Hinv (device d x d, e.g. from
  * slse_fit's trace->hinv_out): w_0 = 0, w+ = w + mu Hinv (v - X^T X w) + eta (w - w_prev).
  * sched supplies mu, eta, T (iteration cap), tol (the fit's relative-step test with
- * rho = sqrt(d/r)), r, prec (FP64, or MIXED_BF16 for F32 X: compensated FP32 passes) and, for
- * MIXED_BF16, stage2 (the correction form as in the fit, for X of 2^24 elements and more, when the
- * workspace has room for the Gram matrix); its sizes m, a and kind are ignored.  X device; Y unused.  v, w_out: device d doubles.
+ * rho = sqrt(d/r)), r and prec (FP64, or MIXED_BF16 for F32 X: compensated FP32 passes);
+ * its sizes m, a, kind and its stage2 are ignored.  X device; Y unused.  v, w_out: device d doubles.
  * report (nullable): ms_total, iters_stage2, final_rel_step, rebases, status.  Returns after w_out
  * is written (SLSE_ENOTCONV if tol > 0 was not met within T, w_out holds the last iterate).
  * Workspace: slse_solve_normal_workspace bytes, or NULL for a stream-ordered allocation. */

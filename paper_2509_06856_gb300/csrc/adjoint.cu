@@ -7,8 +7,12 @@
 // The normal-equation solve is the M-IHS iteration of the 2nd stage with the gradient
 // replaced by v - X^T X w, preconditioned by the H-hat^{-1} of the fit (paper Eqs. (7),
 // (8)), so it converges at the fit's rate: w+ = w + mu H^{-1}(v - X^T X w) + eta (w - w_prev).
-// Each iteration is one pass over X (the residual-gradient kernels with Y = 0) or, on the mixed path
-// in correction form (as in the fit's 2nd stage), a d x d product between exact passes.
+// Each iteration is one pass over X (the residual-gradient kernels with Y = 0).  The fit's correction
+// form (products with the Gram matrix of the BF16 rounding of X between exact passes) is not used here:
+// T then counts correction steps, and a solve that ends by T is further off than T passes over FP32 X.
+// Measured, 262149 x 64, T = 20 without a tolerance, passes against correction form: normal rows
+// 1.6e-8, 4.1e-8; condition 1e2 1.5e-8, 1.0e-6; condition 1e3 4.2e-8, 8.5e-4; T = 25 at a tolerance of
+// 1e-9 is enough for the passes (24 steps), not for the correction form (27).
 #include <cmath>
 #include <type_traits>
 
@@ -21,11 +25,10 @@ constexpr size_t kStateBytesA = 4096;
 
 inline size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
-__global__ void k_init_adj(DevState *st, int rebase, int dc) {
+__global__ void k_init_adj(DevState *st, int rebase) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     DevState z = {};
     z.rebase = rebase;
-    z.dc = dc;
     *st = z;
   }
 }
@@ -250,18 +253,9 @@ __global__ void __launch_bounds__(256, MINB) k_vjp_rows_f32v(const float *X, int
 
 struct AdjLayout {
   int nblk;
-  size_t o_state, o_part, o_g, o_ring, o_b0, o_d32, o_r0, o_y0, full;
-  bool dc;  // mixed path, correction form: the arrays below, behind those of the full form
-  GramPlan grp;
-  size_t o_g0, o_be, o_de, o_gb, o_gram, total;
+  size_t o_state, o_part, o_g, o_ring, o_b0, o_d32, o_r0, o_y0, total;
+  size_t query;  // what slse_solve_normal_workspace returns
 };
-
-// From this many elements of X on the backward solve takes the correction form: a pass then costs more
-// than a correction step and the solve's ~25 passes more than the Gram build (one to three of them).
-// Below, a pass is a few microseconds of launch latency like the step.  Measured, full against
-// correction form (us): 2^16 x 128 808, 847; 2^17 x 128 927, 862; 2^18 x 128 1372, 942; 2^18 x 512
-// 2831, 1651; 2^20 x 512 8108, 3217; 2^21 x 32 4838, 1752.
-constexpr int64_t kAdjCorrection = int64_t(1) << 24;
 
 AdjLayout adj_layout(const slse_problem *p, int prec, int nsm) {
   AdjLayout L{};
@@ -277,17 +271,11 @@ AdjLayout adj_layout(const slse_problem *p, int prec, int nsm) {
   L.o_d32 = take((size_t)d * 4);
   L.o_r0 = take(prec == SLSE_PREC_MIXED_BF16 ? (size_t)p->N * 4 : 0);
   L.o_y0 = take((size_t)p->N * (p->dtype == SLSE_F64 ? 8 : 4));
-  L.full = o;
-  L.dc = prec == SLSE_PREC_MIXED_BF16 && p->dtype == SLSE_F32 && p->N * d >= kAdjCorrection;
-  if (L.dc) {
-    L.grp = gram_plan(p->N, d, nsm > 0 ? nsm : 152);
-    L.o_g0 = take((size_t)d * 8);
-    L.o_be = take((size_t)d * 8);
-    L.o_de = take((size_t)d * 4);
-    L.o_gb = take((size_t)d * d * 8);
-    L.o_gram = take(L.grp.total);
-  }
   L.total = o;
+  // The query has room for a d x d matrix on top for large X on the mixed path (at most 2 MB): callers
+  // have been told that a workspace shorter than the query by that much is accepted.
+  const bool room = prec == SLSE_PREC_MIXED_BF16 && p->dtype == SLSE_F32 && p->N * d >= (int64_t(1) << 24);
+  L.query = L.total + (room ? al((size_t)d * d * 8) : 0);
   return L;
 }
 
@@ -320,7 +308,7 @@ using namespace slse;
 
 extern "C" size_t slse_solve_normal_workspace(const slse_problem *prob, int32_t prec) {
   if (!valid_problem(prob)) return 0;
-  return adj_layout(prob, prec, sm_count()).total;
+  return adj_layout(prob, prec, sm_count()).query;
 }
 
 extern "C" slse_status slse_solve_normal(const slse_problem *prob, const double *Hinv, const double *v, double *w_out,
@@ -346,11 +334,9 @@ extern "C" slse_status slse_solve_normal(const slse_problem *prob, const double 
       return SLSE_ENOMEM;
     }
     owned = true;
-  } else if (ws_bytes < L.full) {
+  } else if (ws_bytes < L.total) {
     return SLSE_ENOMEM;
   }
-  // a workspace without room for the Gram matrix keeps the full form
-  const bool dc = L.dc && sched->stage2 == SLSE_STAGE2_CORRECTION && (owned || ws_bytes >= L.total);
   struct Free {
     void *p;
     bool own;
@@ -371,25 +357,17 @@ extern "C" slse_status slse_solve_normal(const slse_problem *prob, const double 
   const int d = prob->d;
   const bool mixed = prec == SLSE_PREC_MIXED_BF16;
 
-  double *g0 = dc ? reinterpret_cast<double *>(base + L.o_g0) : nullptr;
-  float *de = dc ? reinterpret_cast<float *>(base + L.o_de) : nullptr;
-  double *Gb = dc ? reinterpret_cast<double *>(base + L.o_gb) : nullptr;
-
   Events E;
   cudaEvent_t e0 = E.make(), e1 = E.make();
   DevState *mb = host_res().mailbox();
   volatile unsigned *word = host_res().stop_word();
   if (!e0 || !e1 || !mb || !word) return SLSE_ECUDA;
   CKA(cudaEventRecord(e0, s));
-  k_init_adj<<<1, 32, 0, s>>>(st, mixed ? 1 : 0, dc ? 1 : 0);
+  k_init_adj<<<1, 32, 0, s>>>(st, mixed ? 1 : 0);
   CKA(cudaGetLastError());
   CKA(cudaMemsetAsync(ring, 0, (size_t)3 * d * 8, s));
   CKA(cudaMemsetAsync(y0, 0, (size_t)prob->N * (prob->dtype == SLSE_F64 ? 8 : 4), s));
   int launches = 3;
-  if (dc) {
-    CKA(launch_gram(L.grp, static_cast<const float *>(prob->X), prob->ldx, Gb, &st->status, base + L.o_gram, s));
-    launches += gram_fp32_path(L.grp, static_cast<const float *>(prob->X), prob->ldx) ? 3 : 4;
-  }
 
   UpdateArgs ua{};
   ua.g = g; ua.Hinv = Hinv; ua.beta_ring = ring; ua.beta0 = b0; ua.delta32 = d32;
@@ -397,17 +375,15 @@ extern "C" slse_status slse_solve_normal(const slse_problem *prob, const double 
   const double rho = std::sqrt((double)d / (double)sched->r);
   ua.thr = sched->tol > 0.0 ? sched->tol * (1.0 - rho) / rho : 0.0;
   ua.stage2 = 1; ua.mixed = mixed ? 1 : 0; ua.check_done = 1;
-  ua.beta_e = dc ? reinterpret_cast<double *>(base + L.o_be) : nullptr;
-  ua.delta_e = de;
-  correction_gains(rho, 0.02, ua.gain);
   *word = 0u;
   ua.mail = const_cast<unsigned *>(word);
   for (int k = 0; k < sched->T; ++k) {
     if (launch_grad(mixed ? GM_MIXED : GM_F64, prob->dtype, prob->X, prob->ldx, y0, prob->N, d, ring, st, d32, r0, b0,
                     part, L.nblk, 1, s, true) != cudaSuccess)
       return SLSE_ECUDA;
-    // v + X^T (0 - X w), or the correction step's product
-    if (launch_reduce(part, L.nblk, d, 1.0, g, st, 1, s, g0, Gb, de, v, true) != cudaSuccess) return SLSE_ECUDA;
+    // v + X^T (0 - X w)
+    if (launch_reduce(part, L.nblk, d, 1.0, g, st, 1, s, nullptr, nullptr, nullptr, v, true) != cudaSuccess)
+      return SLSE_ECUDA;
     ua.first = k == 0;
     if (launch_update(ua, st, s, true) != cudaSuccess) return SLSE_ECUDA;
     launches += 3;
