@@ -115,17 +115,22 @@ __device__ __forceinline__ void warp_sum_rows(double (&v)[R], int lane) {
 //  - the row's terms are aligned to the largest exponent F of x_ij beta_j over the row: x_ij's
 //    mantissa becomes the 62-bit integer (zh 2^31 + zl) 2^(F - be ..), bits below 2^-61 of the
 //    row's largest term are dropped;
-//  - zh bh, zh bl and zl bh are summed exactly in 64 bits (three 32 x 32 + 64 bit multiply-adds;
-//    zl bl, at most 2^-58 of the largest term, is left out), the lanes' 96-bit sums are added
-//    exactly in 26-bit pieces, and the total is rounded to FP64 once.
+//  - zh bh, zh bl and zl bh are summed exactly in 64 bits (three 32 x 32 + 64 bit multiply-adds), the
+//    lanes' 96-bit sums are added exactly in 26-bit pieces, and the total is rounded to FP64 once;
+//  - of zl bl the upper 32 bits are summed (FP64 storage; an FP32 mantissa fits zh, but for terms below
+//    2^-7 of the row's largest).  It has the sign of its term: without it every x_i beta came out 2^-59
+//    too small, an error of the gradient along X^T X beta that grew with the rows.  Residual 1e-3 of
+//    X beta, 131072 x 10, error against a double-double sum: FP64 chain 2.6e-13, without zl bl 1.4e-12, with
+//    it 1.8e-13.  It costs 4 % at 2^20 x 256 (with all 64 bits 8 %).
 // The error of x_i beta is then below that of an FP64 chain (2^-53 of the partial sums at each of
 // its d steps): sqrt(d) 2^-60 of the row's largest term, and half an ulp.  A row group with a
 // denormal, an infinity or a NaN, or whose largest product is outside [2^-846, 2^954], takes the FP64
 // sums (warp-uniform).
-// Measured (GB300): N = 2^20, d = 256 FP64 1.07 -> 0.63 ms, d = 512 FP64 2.00 -> 1.17 ms, FP32 storage
-// 2.03 -> 1.23 ms; N = 700001, d = 200 0.725 -> 0.436 ms.  What bounds it now: the FP64 pipe, 0.76
-// busy (the integer pipe 0.67).  Without the ring (rows prefetched into registers) 0.69 ms at 2^20 x
-// 256, without any prefetch 0.86 ms, with three CTAs of 80 registers 0.77 ms.
+// Measured (GB300), the whole call against the FP64 chain: N = 2^20, d = 256 FP64 1.10 -> 0.69 ms, d = 512
+// FP64 2.02 -> 1.25 ms, FP32 storage 2.08 -> 1.25 ms.  What bounds it now: the FP64 pipe, 0.76
+// busy (the integer pipe 0.67).  Before zl bl (0.63 ms at 2^20 x 256): 0.69 ms without
+// the ring (rows prefetched into registers), 0.86 ms without any prefetch, 0.77 ms with three CTAs of
+// 80 registers.
 struct BetaFix {
   int bh, bl, be;
 };
@@ -144,6 +149,11 @@ __device__ __forceinline__ BetaFix beta_fix(double b) {
 // a + b c, signed 32 x 32 bits into 64
 __device__ __forceinline__ long long madw(int b, int c, long long a) {
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a) : "r"(b), "r"(c));
+  return a;
+}
+// a + the upper 32 bits of b c
+__device__ __forceinline__ int madh(int b, int c, int a) {
+  asm("mad.hi.s32 %0, %1, %2, %0;" : "+r"(a) : "r"(b), "r"(c));
   return a;
 }
 // logical right shift that gives 0 from 32 on (the C operator does not define it)
@@ -311,6 +321,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_grad_f64(const GradArgs a) 
         }
       fmax = __reduce_max_sync(0xffffffffu, fmax);
       long long sh = 0, s1 = 0, s2 = 0;
+      int s3 = 0;
 #pragma unroll
       for (int v = 0; v < VMAX; ++v)
 #pragma unroll
@@ -328,7 +339,9 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_grad_f64(const GradArgs a) 
           sh = madw(zh, b.x, sh);
           s1 = madw(zl, b.x, s1);
           s2 = madw(zh, b.y, s2);
+          if constexpr (sizeof(Tx) == 8) s3 = madh(zl, b.y, s3);
         }
+      s1 += (long long)s3 << 6;
       // sh 2^31 + s1 + s2 2^5, in 96 bits
       const uint32_t hl = (uint32_t)sh, hh = (uint32_t)(sh >> 32);
       uint32_t w0 = hl << 31, w1 = __funnelshift_l(hl, hh, 31), w2 = (uint32_t)((int)hh >> 1);
