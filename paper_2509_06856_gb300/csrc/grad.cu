@@ -125,7 +125,9 @@ __device__ __forceinline__ void warp_sum_rows(double (&v)[R], int lane) {
 // The error of x_i beta is then below that of an FP64 chain (2^-53 of the partial sums at each of
 // its d steps): sqrt(d) 2^-60 of the row's largest term, and half an ulp.  A row group with a
 // denormal, an infinity or a NaN, or whose largest product is outside [2^-846, 2^954], takes the FP64
-// sums (warp-uniform).
+// sums (warp-uniform).  A row without a non-zero term has the sum zero and stays here (in
+// the FP64 sums, which read X again element by element, a pass at beta = 0 took 2420 us at 2^20 x 512, FP32
+// storage 3390; now 1190 and 1180).
 // Measured (GB300), the whole call against the FP64 chain: N = 2^20, d = 256 FP64 1.10 -> 0.69 ms, d = 512
 // FP64 2.02 -> 1.25 ms, FP32 storage 2.08 -> 1.25 ms.  What bounds it now: the FP64 pipe, 0.76
 // busy (the integer pipe 0.67).  Before zl bl (0.63 ms at 2^20 x 256): 0.69 ms without
@@ -362,8 +364,9 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_grad_f64(const GradArgs a) 
     const bool rv = lane < RPW && i0 + lane < a.nrows;
     odd = __any_sync(0xffffffffu, odd);
     double r[RPW];
-    if (!beta_odd && !odd && !__any_sync(0xffffffffu, rv && (uint32_t)(F - 1200) > 1800u)) {
-      const double rl = rv ? y - dot_total(p0, p1, p2, p3, F) : 0.0;
+    const bool none = F < kNoTerm / 2;  // no non-zero term: a row of zeros, or beta = 0
+    if (!beta_odd && !odd && !__any_sync(0xffffffffu, rv && !none && (uint32_t)(F - 1200) > 1800u)) {
+      const double rl = rv ? (none ? y : y - dot_total(p0, p1, p2, p3, F)) : 0.0;
 #pragma unroll
       for (int q = 0; q < RPW; ++q) r[q] = __shfl_sync(0xffffffffu, rl, q);
     } else {
