@@ -614,30 +614,21 @@ void gram_f32_layout(int ncp, const GramRole *ro, int Q, GramF32Args &a, size_t 
 // X (the same relative rounding, 2^-9 per element), at half the bytes and with no rounding work:
 // the MMA reads W's row-major tiles as MN-major operands straight from the TMA boxes (64 columns x
 // 64 rows, 128-byte swizzle).
-// Roles as in k_gram_f32 (the same tiles); each 64-column box of a stage is loaded once by one CTA
-// and multicast to the CTAs whose tiles read it, the loads spread over the cluster:
-//   ncp 512: boxes 0-3 -> {r0, r1}: r1 loads 0, 1, 2, r0 loads 3; boxes 4-7 -> {r0, r2}: r2 loads
-//            4, 5, 6, r0 loads 7
-//   ncp 384: boxes 0-1 -> {r0}: r0 loads; boxes 2-5 -> {r0, r1}: r1 loads 2, 3, 4, r0 loads 5
-//   ncp <= 256: one CTA loads every box
-// A CTA releases a stage's buffer (its incoming bytes expected, the loaders of its boxes told) once
-// its MMAs of the stage that used the buffer before have completed; a loader issues a stage's
-// boxes once every destination has released the buffer.
+// Roles as in k_gram_f32 (the same tiles), one CTA per role, not in a cluster: each loads the
+// 64-column boxes that its tiles read.  The CTAs of a range run side by side, so the second reader of a
+// box mostly finds it in L2; sharing each box over a cluster measured 1.8x slower at d = 512 (3.28 against
+// 1.83 ms at N = 2^22: the CTAs' buffer hand-offs serialised the stages).
+// A buffer is released (its incoming bytes expected, the load warp told) once the MMAs of the stage
+// that used it before have completed.
 // rows of B per stage: KR = 64 (4 K steps; 32-row stages, twice as many in flight, measured 1.7x
 // slower at d = 512); a box is 64 columns x KR rows (KR 128 bytes)
-// boxes multicast within a cluster (each loaded once) or loaded by every CTA that reads them: the
-// latter measured 1.8x faster at d = 512 (1.83 against 3.28 ms at N = 2^22; the cluster's
-// buffer hand-offs serialised the stages), so multicast is kept only as the other form of the roles
-constexpr bool kWMulticast = false;
 constexpr int kWThreads = 224;           // warp 0: loads, warp 1: MMAs, warp 2: releases, warps 3-6: epilogue
 
 struct GramWRole {
   int ntile;
   int a_blk[2], b_lo[2], n[2], toff[2];
-  uint32_t issue;      // bit j: this CTA loads box j
-  uint32_t feeds;      // bit q: CTA q loads boxes this CTA reads (it is told of releases)
-  int nfree;           // number of CTAs a release of this CTA's loads waits for
-  int recv_bytes;      // bytes this CTA receives per stage
+  uint32_t issue;      // bit j: this CTA reads box j
+  int recv_bytes;      // bytes of those boxes
 };
 
 struct GramWArgs {
@@ -647,8 +638,6 @@ struct GramWArgs {
   int64_t nstage, cps;
   int ncp, nbox, tmem_cols, Q, S;
   int o_bar;
-  uint16_t dest[8];    // CTA mask receiving box j (multicast)
-  int mc;              // boxes multicast within the cluster (else every CTA loads its own)
   GramWRole role[3];
 };
 
@@ -658,28 +647,19 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr, uint32_t lbo
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
          (1ull << 46) | (2ull << 61);
 }
-// 2-D TMA load multicast to the CTAs of mask (the same shared offset and mbarrier in each)
-__device__ __forceinline__ void tma_load_2d_mc(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar,
-                                               uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, "
-      "{%2, %3}], [%4], %5;" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar)), "h"(mask)
-      : "memory");
-}
 
 template <int KR>
 __global__ void __launch_bounds__(kWThreads, 1) k_gram_w(const __grid_constant__ GramWArgs a) {
   constexpr uint32_t kBox = KR * 128;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int rank = (int)blockIdx.x;  // cluster (Q, 1, 1) over grid (Q, ranges)
+  const int rank = (int)blockIdx.x;  // role; grid (Q, ranges)
   const GramWRole ro = rank == 0 ? a.role[0] : (rank == 1 ? a.role[1] : a.role[2]);
   const int S = a.S;
   const uint32_t bstage = (uint32_t)a.nbox * kBox;
   uint64_t *full = reinterpret_cast<uint64_t *>(sm + a.o_bar);
   uint64_t *empty = full + kFMaxB;
-  uint64_t *slotfree = empty + kFMaxB;  // the destinations of this CTA's loads released a buffer
+  uint64_t *slotfree = empty + kFMaxB;  // a buffer is released
   uint64_t *accum = slotfree + kFMaxB;
   uint32_t *tslot = reinterpret_cast<uint32_t *>(accum + 1);
   volatile int *abort_f = reinterpret_cast<volatile int *>(tslot + 1);
@@ -691,7 +671,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_gram_w(const __grid_constant__
     for (int s = 0; s < S; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
-      mbar_init(&slotfree[s], ro.nfree > 0 ? ro.nfree : 1);
+      mbar_init(&slotfree[s], 1);
     }
     mbar_init(accum, 1);
     *abort_f = 0;
@@ -707,8 +687,6 @@ __global__ void __launch_bounds__(kWThreads, 1) k_gram_w(const __grid_constant__
   }
   tc_fence_before();
   __syncthreads();
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   tc_fence_after();
   const uint32_t tmem = *tslot;
   const int64_t st0 = (int64_t)blockIdx.y * a.cps;
@@ -716,7 +694,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_gram_w(const __grid_constant__
   const int nk = (int)(st1 - st0);
 
   if (warp == 0) {
-    if (lane == 0 && ro.issue != 0u) {
+    if (lane == 0) {
       for (int k = 0; k < nk; ++k) {
         const int s = k % S;
         if (!mbar_wait(&slotfree[s], (uint32_t)(k / S) & 1u, abort_f, a.status)) break;
@@ -724,8 +702,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_gram_w(const __grid_constant__
         for (int j = 0; j < a.nbox; ++j) {
           if (!(ro.issue >> j & 1u)) continue;
           uint8_t *dst = sm + (size_t)s * bstage + (size_t)j * kBox;
-          if (!a.mc) tma_load_2d(dst, &a.tmap, 64 * j, y, &full[s]);
-          else tma_load_2d_mc(dst, &a.tmap, 64 * j, y, &full[s], a.dest[j]);
+          tma_load_2d(dst, &a.tmap, 64 * j, y, &full[s]);
         }
       }
     }
@@ -760,7 +737,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_gram_w(const __grid_constant__
       *s_consumed = consumed;
     }
   } else if (warp == 2) {
-    // releases: buffer s for stage j (its incoming bytes expected, its loaders told) once the MMAs
+    // releases: buffer s for stage j (its incoming bytes expected, the load warp told) once the MMAs
     // of stage j - S have completed
     if (lane == 0) {
       int released = 0;
@@ -768,11 +745,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_gram_w(const __grid_constant__
         const int s = j % S;
         if (j >= S && !mbar_wait(&empty[s], (uint32_t)((j - S) / S) & 1u, abort_f, a.status)) break;
         mbar_arrive_expect_tx(&full[s], (uint32_t)ro.recv_bytes);
-        for (int q = 0; q < a.Q; ++q) {
-          if (!(ro.feeds >> q & 1u)) continue;
-          if (q == rank) mbar_arrive(&slotfree[s]);
-          else mbar_arrive_remote(cluster_addr(smem_u32(&slotfree[s]), q));
-        }
+        mbar_arrive(&slotfree[s]);
         released = j + 1;
       }
       *s_released = released;
@@ -807,12 +780,10 @@ __global__ void __launch_bounds__(kWThreads, 1) k_gram_w(const __grid_constant__
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols) : "memory");
   }
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // roles of k_gram_w for ncp columns (the table above it); returns Q
-int gram_w_roles(int ncp, int box_bytes, GramWArgs &a, bool multicast) {
+int gram_w_roles(int ncp, int box_bytes, GramWArgs &a) {
   GramRole cr[3];
   const int Q = gram_roles(ncp, cr, nullptr);
   a.Q = Q;
@@ -829,41 +800,13 @@ int gram_w_roles(int ncp, int box_bytes, GramWArgs &a, bool multicast) {
       w.toff[t] = cr[r].toff[t];
     }
   }
-  a.mc = multicast && Q > 1 ? 1 : 0;
-  for (int j = 0; j < 8; ++j) a.dest[j] = 0;
-  if (!a.mc) {
-    // every CTA loads the boxes its tiles read (the CTAs of a range run side by side, so the
-    // second reader of a box mostly finds it in L2)
-    for (int r = 0; r < Q; ++r) {
-      GramWRole &w = a.role[r];
-      for (int t = 0; t < w.ntile; ++t) {
-        for (int c = kGM * w.a_blk[t]; c < kGM * (w.a_blk[t] + 1); c += 64) w.issue |= 1u << (c / 64);
-        for (int c = w.b_lo[t]; c < w.b_lo[t] + w.n[t]; c += 64) w.issue |= 1u << (c / 64);
-      }
-      w.feeds = 1u << r;
-      w.nfree = 1;
-      w.recv_bytes = __builtin_popcount(w.issue) * box_bytes;
-    }
-    return Q;
-  }
-  uint32_t issuer[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  if (Q == 1) {
-    for (int j = 0; j < a.nbox; ++j) { a.dest[j] = 1; issuer[j] = 0; }
-  } else if (Q == 2) {
-    const int iss[6] = {0, 0, 1, 1, 1, 0};
-    for (int j = 0; j < 6; ++j) { a.dest[j] = j < 2 ? 0x1 : 0x3; issuer[j] = (uint32_t)iss[j]; }
-  } else {
-    const int iss[8] = {1, 1, 1, 0, 2, 2, 2, 0};
-    for (int j = 0; j < 8; ++j) { a.dest[j] = j < 4 ? 0x3 : 0x5; issuer[j] = (uint32_t)iss[j]; }
-  }
   for (int r = 0; r < Q; ++r) {
     GramWRole &w = a.role[r];
-    uint32_t dests = 0;
-    for (int j = 0; j < a.nbox; ++j) {
-      if ((int)issuer[j] == r) { w.issue |= 1u << j; dests |= a.dest[j]; }
-      if (a.dest[j] >> r & 1u) { w.recv_bytes += box_bytes; w.feeds |= 1u << issuer[j]; }
+    for (int t = 0; t < w.ntile; ++t) {
+      for (int c = kGM * w.a_blk[t]; c < kGM * (w.a_blk[t] + 1); c += 64) w.issue |= 1u << (c / 64);
+      for (int c = w.b_lo[t]; c < w.b_lo[t] + w.n[t]; c += 64) w.issue |= 1u << (c / 64);
     }
-    w.nfree = __builtin_popcount(dests);
+    w.recv_bytes = __builtin_popcount(w.issue) * box_bytes;
   }
   return Q;
 }
@@ -1009,7 +952,7 @@ GramWPlan gram_w_plan(int64_t rows, int d, int nsm) {
   p.tmem_cols = tc;
   GramWArgs a{};
   p.kr = 64;
-  const int Q = gram_w_roles(p.ncp, p.kr * 128, a, kWMulticast);
+  const int Q = gram_w_roles(p.ncp, p.kr * 128, a);
   p.q = Q;
   p.nstage = gcdiv(rows, p.kr);
   gram_split(p.nstage, Q, nsm, p.cps, p.splits, 8192 / p.kr);
@@ -1055,25 +998,14 @@ cudaError_t launch_gram_w(const GramWPlan &p, const void *B, int64_t ldb, double
   a.cps = p.cps;
   a.ncp = p.ncp;
   a.tmem_cols = p.tmem_cols;
-  gram_w_roles(p.ncp, p.kr * 128, a, kWMulticast);
+  gram_w_roles(p.ncp, p.kr * 128, a);
   size_t smem = 0;
   gram_w_layout(p.ncp, p.kr, a, smem);
   cudaError_t e;
   auto kern = p.kr == 32 ? k_gram_w<32> : k_gram_w<64>;
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)a.Q, (unsigned)p.splits);
-  cfg.blockDim = dim3(kWThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = a.mc ? (unsigned)a.Q : 1u;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if ((e = cudaLaunchKernelEx(&cfg, kern, a))) return e;
+  kern<<<dim3((unsigned)a.Q, (unsigned)p.splits), kWThreads, smem, s>>>(a);
+  if ((e = cudaGetLastError())) return e;
   return launch_gram_reduce(part, p.splits, p.ncp, p.d, scale,
                             reinterpret_cast<double *>(reinterpret_cast<char *>(part) + p.o_grp), status, G, s);
 }
