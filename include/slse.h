@@ -207,7 +207,8 @@ slse_status slse_fit(const slse_problem *prob, const slse_schedule *sched, uint6
  * device wait that gave up leaves NaN in SX and SY.  prec FP64 ->
  * SX, SY are double; MIXED_BF16 -> bf16 (CountSketch sums accumulated in FP32, in row
  * order within a bucket, so the result is deterministic).  SX: device m x ldsx (ldsx >= d),
- * SY: device m.  prec MIXED_FP8 (kind SRHT): SX holds m x ldsx E4M3 bytes (ldsx a multiple of
+ * SY: device m.  kind SLSE_SRHT: a bounded device wait that gave up leaves NaN in SX and SY, as above.
+ * prec MIXED_FP8 (kind SRHT): SX holds m x ldsx E4M3 bytes (ldsx a multiple of
  * 4, SX 4-byte aligned) followed by m x ceil(d/32) block-exponent bytes; SY is bf16.
  * Asynchronous on `stream`; the workspace size comes from
  * slse_workspace_size(SLSE_OP_SKETCH) with sched->kind and sched->prec set. */
@@ -325,10 +326,10 @@ const char *slse_status_string(int32_t status);
 /* Fault injection for tests (no paper counterpart).  Sets how many polls a grid-wide wait of
  * the library (the grid barrier of the FP64 Householder QR, slse_qr and the FP64 fit) makes
  * before it gives up; the call then reports SLSE_ETIMEOUT and every CTA of the grid stops at
- * that barrier or the next.  polls <= 0 restores the built-in limit (2^25 polls, about a
+ * that barrier or the next.  The waits within a CTA of the SRHT's tensor-core passes follow it too.  polls <= 0 restores the built-in limit (2^25 polls, about a
  * second).  Process-wide; takes effect for calls started afterwards.  Returns the previous
- * setting (0 = built-in).  The mbarrier waits of the tensor-core kernel keep their own fixed
- * time limit. */
+ * setting (0 = built-in).  The mbarrier waits of the other tensor-core kernels keep their own
+ * fixed time limit. */
 int64_t slse_debug_spin_limit(int64_t polls);
 
 /* Library version: major*10000 + minor*100 + patch. */

@@ -971,6 +971,12 @@ slse_status slse_sketch(const slse_problem *prob, int32_t kind, int32_t prec, ui
   int32_t *pos = reinterpret_cast<int32_t *>(base + L.o_pos);
   CK(launch_draws(Np, seed, Psd, nullptr, sigma, nullptr, base + L.o_big, st));
   CK(launch_pos_map(sigma, Np, 0, m, L.sp.single ? L.sp.logN : L.sp.log2, pos, st));
+  // sigma is not read any more: its first word takes the passes' status (a wait that gave up leaves NaN)
+  unsigned *status = nullptr;
+  if (!L.sp.single) {
+    status = reinterpret_cast<unsigned *>(sigma);
+    CK(cudaMemsetAsync(status, 0, sizeof(unsigned), st));
+  }
   if (prec == SLSE_PREC_MIXED_FP8) {
     // SX: m x ldsx E4M3 bytes followed by the m x ceil(d/32) block-exponent bytes
     uint8_t *scales = static_cast<uint8_t *>(SX) + (size_t)m * ldsx;
@@ -982,12 +988,14 @@ slse_status slse_sketch(const slse_problem *prob, int32_t kind, int32_t prec, ui
                             static_cast<uint8_t *>(SX), ldsx, scales, nsb, st));
     } else {
       CK(launch_srht(L.sp, prec, prob->dtype, prob->X, prob->ldx, prob->Y, prob->N, prob->d, Psd, pos, base + L.o_big,
-                     base + L.o_wy, L.ldw, SX, SY, ldsx, 1.0 / std::sqrt((double)m), st, nullptr, scales, nsb));
+                     base + L.o_wy, L.ldw, SX, SY, ldsx, 1.0 / std::sqrt((double)m), st, nullptr, scales, nsb, nullptr,
+                     0, 0, nullptr, status));
     }
     return SLSE_OK;
   }
   CK(launch_srht(L.sp, prec, prob->dtype, prob->X, prob->ldx, prob->Y, prob->N, prob->d, Psd, pos, base + L.o_big,
-                 base + L.o_wy, L.ldw, SX, SY, ldsx, 1.0 / std::sqrt((double)m), st, nullptr));
+                 base + L.o_wy, L.ldw, SX, SY, ldsx, 1.0 / std::sqrt((double)m), st, nullptr, nullptr, 0, nullptr, 0, 0,
+                 nullptr, status));
   return SLSE_OK;
 }
 

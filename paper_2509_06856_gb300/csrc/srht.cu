@@ -32,6 +32,8 @@
 #include <cooperative_groups.h>
 #include <cuda_fp8.h>
 
+#include <math_constants.h>
+
 #include <type_traits>
 
 #include "srht_args.cuh"
@@ -360,8 +362,8 @@ __global__ void __launch_bounds__(NT, MINB) k_group(const GroupArgs a) {
   // stage O: tile ready.  The CTA barrier orders every thread's tile stores before thread 0's
   // single cluster-scope release fence; thread 0 then signals each peer's barrier, and every
   // thread waits, with acquire, until all Q tiles of the cluster are ready.  The wait gives up
-  // after ~2^22 polls (ST_TIMEOUT; the output is then garbage but no CTA leaves before its
-  // peers, so no remote read outlives its tile).
+  // after ~2^22 polls (ST_TIMEOUT, see k_ycol; no CTA leaves before its peers, so no remote read
+  // outlives its tile).
   __syncthreads();
   if constexpr (Q > 1) {
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // the peers' barriers are initialised
@@ -471,10 +473,23 @@ __global__ void __launch_bounds__(NT, MINB) k_group(const GroupArgs a) {
   }
 }
 
+// NaN in output row dst of the X columns
+template <class TX> __device__ __noinline__ void mark_row(const GroupArgs &a, int64_t dst) {
+  for (int c = 0; c < a.d; ++c) {
+    if constexpr (std::is_same_v<TX, mx8>) {
+      if (a.hat_out && dst >= a.hat_row0) store_cvt(a.hat_out + (dst - a.hat_row0) * a.hat_ld + c, CUDART_NAN_F);
+      else static_cast<uint8_t *>(a.out)[dst * a.ldout + c] = 0x7F;
+    } else {
+      store_cvt(static_cast<TX *>(a.out) + dst * a.ldout + c, CUDART_NAN_F);
+    }
+  }
+}
+
 // The Y column of one group (2^L <= 4096 rows) per CTA, in shared memory: gather
 // (with signs) or strided read, butterflies level by level, scaled store to the
-// sampled rows.
-template <class Tin, class Ts, class Tout>
+// sampled rows.  It runs behind the X columns' kernel (whose outputs are TX): where a wait of a pass gave
+// up, the last pass leaves NaN in the sampled rows, whose values are then not the sketch.
+template <class Tin, class Ts, class Tout, class TX>
 __global__ void __launch_bounds__(512) k_ycol(const GroupArgs a, int L) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Ts *t = reinterpret_cast<Ts *>(smem_raw);
@@ -505,10 +520,13 @@ __global__ void __launch_bounds__(512) k_ycol(const GroupArgs a, int L) {
     __syncthreads();
   }
   Tout *out_y = static_cast<Tout *>(a.out_y);
+  const bool bad = a.pos && a.status && (*(volatile const unsigned *)a.status & ST_TIMEOUT) != 0;
   for (int kap = threadIdx.x; kap < n; kap += blockDim.x) {
     const int64_t k = out_row(a, kap, g);
     const int64_t dst = a.pos ? (int64_t)__ldg(a.pos + k) : k;
-    if (dst >= 0) store_cvt(out_y + dst, t[kap] * (Ts)a.scale);
+    if (dst < 0) continue;
+    if (bad) mark_row<TX>(a, dst);
+    store_cvt(out_y + dst, bad ? Ts(CUDART_NAN_F) : t[kap] * (Ts)a.scale);
   }
 }
 
@@ -650,7 +668,7 @@ cudaError_t launch_pass_t(const GroupArgs &a, int L, int64_t ngroups, cudaStream
   if (e != cudaSuccess) return e;
   const size_t ysm = (size_t)(1 << L) * sizeof(Ts);
   using TY = std::conditional_t<std::is_same_v<Tout, mx8>, __nv_bfloat16, Tout>;  // FP8 form: Y in BF16
-  auto ykern = k_ycol<Tin, Ts, TY>;
+  auto ykern = k_ycol<Tin, Ts, TY, Tout>;
   if ((e = cudaFuncSetAttribute(ykern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ysm)) != cudaSuccess) return e;
   ykern<<<(unsigned)ngroups, 512, ysm, s>>>(a, L);
   return cudaGetLastError();
@@ -677,6 +695,7 @@ cudaError_t run_plan(const SrhtPlan &pl, const void *X, int64_t ldx, const void 
                      int64_t hat_row0 = 0, int64_t hat_ld = 0, void *copy_out = nullptr, unsigned *status = nullptr) {
   GroupArgs a = {};
   a.status = status;
+  a.wait_polls = debug_spin_limit();
   a.d = d;
   a.nslab = (d + 1 + C - 1) / C;
   auto vec_ok = [](const void *p, int64_t ld, size_t eb, int v) {

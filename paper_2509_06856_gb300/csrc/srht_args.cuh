@@ -33,6 +33,7 @@ struct GroupArgs {
   void *copy_out;       // pass 1 reading host memory: every input row segment is also stored
                         // here at the same element offset (the device copy of X)
   unsigned *status;     // nullable: ST_TIMEOUT is raised here when a bounded wait gave up
+  long long wait_polls; // tensor-core form: polls of a wait before it gives up (0: the built-in time limit)
 };
 
 __host__ __device__ __forceinline__ int64_t in_row(const GroupArgs &a, int64_t rho, int64_t g) {

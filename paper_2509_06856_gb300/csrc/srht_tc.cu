@@ -28,8 +28,8 @@
 // alone would take 2.2 ms).  Tried on the way: eight producer warps loading into registers (32 KB on their way
 // per SM: 3.39 ms at 3000000 x 384, 2.24 ms now), eight epilogue warps, H as an MN-major operand (the MMAs ran at
 // half the rate), all output rows read back before the first store (spills).
-// Every mbarrier wait is bounded (ST_TIMEOUT); copies in flight are awaited and tensor memory is
-// freed on that path too.
+// Every mbarrier wait is bounded (ST_TIMEOUT: the fit reports it, slse_sketch's output is NaN then);
+// copies in flight are awaited and tensor memory is freed on that path too.
 #include "srht_args.cuh"
 #include "tc_common.cuh"
 
@@ -148,7 +148,9 @@ __device__ __noinline__ void split3_rare(const float4 x, uint32_t sg, uint2 &h, 
   l = make_uint2(w[2][0] | (w[2][1] << 16), w[2][2] | (w[2][3] << 16));
 }
 
-template <bool F32, int L>
+// POLLS: a test has set a limit to the waits (a form of its own: the test of the limit in every wait cost
+// 30 us of 3.65 ms at 3000000 x 384)
+template <bool F32, int L, bool POLLS>
 __global__ void __launch_bounds__(kTcThreads, 1) k_group_tc(const TcPassArgs A) {
   constexpr int J = 1 << (L - 7);      // rows jh
   constexpr int C = 512 / J;           // columns of a group
@@ -206,10 +208,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_group_tc(const TcPassArgs A) 
   const uint32_t tmem = *tslot;
   const int ntile = (int)((A.ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x);  // of this CTA
   const int nchunk = ntile * kKSteps;
-  // a wait of a whole warp, with one result for all lanes
-  auto wait_all = [&](uint64_t *bar, uint32_t parity) -> bool {
-    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_f, status));
+  auto wait_one = [&](uint64_t *bar, uint32_t parity) -> bool {
+    if constexpr (POLLS) return mbar_wait_polls(bar, parity, abort_f, status, a.wait_polls);
+    else return mbar_wait(bar, parity, abort_f, status);
   };
+  // a wait of a whole warp, with one result for all lanes
+  auto wait_all = [&](uint64_t *bar, uint32_t parity) -> bool { return __all_sync(0xFFFFFFFFu, wait_one(bar, parity)); };
   auto tile_of = [&](int it, int64_t &g, int &col0) {
     const uint32_t item = blockIdx.x + (uint32_t)it * gridDim.x, gg = item / (uint32_t)a.nslab;
     g = (int64_t)gg;
@@ -380,11 +384,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_group_tc(const TcPassArgs A) 
       const uint32_t hb = smem_u32(sm);
       bool ok = true;
       for (int it = 0; it < ntile && ok; ++it) {
-        if (it > 0 && !mbar_wait(tempty, (uint32_t)(it - 1) & 1u, abort_f, status)) break;
+        if (it > 0 && !wait_one(tempty, (uint32_t)(it - 1) & 1u)) break;
         tc_fence_after();
         for (int ks = 0; ks < kKSteps; ++ks) {
           const int n = it * kKSteps + ks, st = n % NST;
-          if (!mbar_wait(&full[st], (uint32_t)(n / NST) & 1u, abort_f, status)) {
+          if (!wait_one(&full[st], (uint32_t)(n / NST) & 1u)) {
             ok = false;
             break;
           }
@@ -566,7 +570,7 @@ template <bool F32, int L> cudaError_t launch_tc(const GroupArgs &a0, int64_t ng
   A.ntiles = ngroups * A.a.nslab;
   const size_t smem = 1024 + kHBytes + (size_t)ring_stages<F32>() * stage_bytes<F32>() + (F32 ? kRaw * kRawBytes : 0) + 8 * (2 * ring_stages<F32>() + 3) + 32 +
                       (F32 ? 0 : 8 * (size_t)(1 << L));
-  auto kern = k_group_tc<F32, L>;
+  auto kern = a0.wait_polls > 0 ? k_group_tc<F32, L, true> : k_group_tc<F32, L, false>;
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)(A.ntiles < nsm ? A.ntiles : nsm), kTcThreads, smem, s>>>(A);

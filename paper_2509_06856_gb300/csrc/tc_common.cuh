@@ -54,6 +54,25 @@ __device__ __noinline__ bool mbar_wait_slow(uint64_t *bar, uint32_t parity, vola
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_f, unsigned *status) {
   return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity, abort_f, status);
 }
+// The same, giving up after `polls` polls (kernels that a test gives a limit).
+__device__ __noinline__ bool mbar_wait_polls(uint64_t *bar, uint32_t parity, volatile int *abort_f, unsigned *status,
+                                             long long polls) {
+  for (long long it = 0;; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok != 0) return true;
+    if (*abort_f) return false;
+    if (it >= polls) {
+      *abort_f = 1;
+      atomicOr(status, ST_TIMEOUT);
+      return false;
+    }
+  }
+}
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
