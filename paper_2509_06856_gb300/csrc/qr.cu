@@ -375,12 +375,22 @@ cudaError_t launch_qr_panels(const double *A, int64_t r, int d, int64_t lda, dou
   // priority; the update of the columns behind those runs beside the next panel on the caller's
   // stream.  Reflectors are double-buffered: block p is read until the update of block p + 1 starts.
   Events E;
-  cudaEvent_t e_chain = E.make(), e_rest = E.make();
-  if (!e_chain || !e_rest) return cudaErrorUnknown;
+  cudaEvent_t e_chain = nullptr, e_rest = nullptr;
   SideStream chain;
-  const bool ahead = d > 2 * kNb;
+  // One stream while the caller's is being captured (a stream of the thread's would stay part of the
+  // capture after the call), and when every side stream has other work.
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+    cudaGetLastError();
+    capture = cudaStreamCaptureStatusActive;
+  }
+  if (d > 2 * kNb && capture == cudaStreamCaptureStatusNone && (e = chain.open(true, s, true)) != cudaSuccess) return e;
+  const bool ahead = chain.h != nullptr;
   if (ahead) {
-    if ((e = chain.open(true, s)) || (e = cudaEventRecord(e_rest, s))) return e;
+    e_chain = E.make();
+    e_rest = E.make();
+    if (!e_chain || !e_rest) return cudaErrorUnknown;
+    if ((e = cudaEventRecord(e_rest, s))) return e;
   }
   const cudaStream_t sc = ahead ? chain.h : s;
   for (int j0 = 0, blk = 0; j0 < d; j0 += kNb, blk ^= 1) {
