@@ -523,7 +523,7 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
     CK(launch_countsketch(L.csp, p->dtype, p->X, p->ldx, p->Y, seed, lvX, lvY, L.ldu,
                           static_cast<char *>(U) + (size_t)L.h0 * L.ldu * eu, static_cast<char *>(V) + (size_t)L.h0 * eu,
                           L.ldu, big, st));
-    kernels += 12;
+    kernels += cs_kernels(L.csp);
     CK(cudaEventRecord(e_mid, st));
   } else {
     // a1: random draws (none when nothing is sampled: a Gaussian Hessian sketch without subproblems)
@@ -598,7 +598,7 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
       kernels += 3;  // Gram, group sums, final sum
     } else {
       e = launch_gram(L.grp, static_cast<const float *>(p->X), p->ldx, Gb, gram_status, big, gram_side.h);
-      kernels += gram_fp32_path(L.grp, static_cast<const float *>(p->X), p->ldx) ? 2 : 3;  // (pack,) Gram, reduce
+      kernels += gram_fp32_path(L.grp, static_cast<const float *>(p->X), p->ldx) ? 3 : 4;  // (pack,) Gram, sums
     }
     if (e) return e;
     return cudaEventRecord(e_gram1, gram_side.h);
@@ -660,8 +660,7 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
                                     std::sqrt(hat_scale2), A, st));
       ++kernels;
     }
-    CK(launch_qr(A, s.r, d, d, R, Hinv, qrws, s.prec == SLSE_PREC_FP64 ? big : nullptr, dst, st));
-    kernels += 3;
+    CK(launch_qr(A, s.r, d, d, R, Hinv, qrws, s.prec == SLSE_PREC_FP64 ? big : nullptr, dst, st, kernels));
   }
   CK(cudaEventRecord(e_qr, st));
   CK(fork_gram(e_qr));
@@ -1087,7 +1086,8 @@ slse_status slse_qr(const double *A, int64_t r, int32_t d, int64_t lda, double *
   k_init_state<<<1, 32, 0, st>>>(dst, 0, debug_spin_limit());
   CK(cudaGetLastError());
   CK(cudaMemcpy2DAsync(Ac, (size_t)d * 8, A, (size_t)lda * 8, (size_t)d * 8, (size_t)r, cudaMemcpyDeviceToDevice, st));
-  CK(launch_qr(Ac, r, d, d, R, Hinv, base + o_qr, panels ? base + o_qrp : nullptr, dst, st));
+  int launched = 0;
+  CK(launch_qr(Ac, r, d, d, R, Hinv, base + o_qr, panels ? base + o_qrp : nullptr, dst, st, launched));
   return SLSE_OK;
 }
 

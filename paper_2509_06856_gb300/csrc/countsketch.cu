@@ -632,6 +632,11 @@ cudaError_t run_cs(const CsPlan &pl, const void *X, int64_t ldx, const void *Y, 
 
 }  // namespace
 
+int cs_kernels(const CsPlan &pl) {
+  const int top = pl.L - pl.F;
+  return 4 + (pl.L >= 0 ? 2 + (top > pl.l1 ? top - pl.l1 : 0) : 0) + (pl.r > 0 ? 2 : 0);
+}
+
 cudaError_t launch_countsketch(const CsPlan &pl, int xdtype, const void *X, int64_t ldx, const void *Y, uint64_t seed,
                                void *const *lvX, void *const *lvY, int64_t ldo, void *hatX, void *hatY, int64_t ldh,
                                void *ws, cudaStream_t s) {

@@ -439,9 +439,9 @@ cudaError_t launch_gather_hessian_rows(int prec, const void *U, int64_t ldu, int
 }
 
 // A is overwritten (it must be a scratch copy).  ws: qr_ws_bytes(r, d); panels: qr_panels_ws_bytes(r, d)
-// or nullptr (column by column).
+// or nullptr (column by column).  Adds the kernels it launches to `launched`.
 cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, double *Hinv, void *ws, void *panels,
-                      DevState *st, cudaStream_t s) {
+                      DevState *st, cudaStream_t s, int &launched) {
   int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -465,7 +465,7 @@ cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, doubl
   // by panels up to 16384 rows (their rows stay in a cluster's registers); the column-by-column form
   // above that, and when a test limits the polls of its grid barrier (the panels have no such wait)
   if (panels && qr_panels_ok(r) && debug_spin_limit() == 0) {
-    if ((e = launch_qr_panels(A, r, d, lda, R, a.Rt, panels, st, s)) != cudaSuccess) return e;
+    if ((e = launch_qr_panels(A, r, d, lda, R, a.Rt, panels, st, s, launched)) != cudaSuccess) return e;
   } else {
     const int64_t nr_max = (r + G - 1) / G;
     const size_t smem = (size_t)nr_max * d * sizeof(double);
@@ -483,11 +483,13 @@ cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, doubl
     void *args[] = {&a};
     e = cudaLaunchCooperativeKernel((const void *)kern, dim3(G), dim3(kQrThreads), args, dyn, s);
     if (e != cudaSuccess) return e;
+    ++launched;
   }
   if (Hinv) {
     k_tri_inv_sweep<<<(d + 7) / 8, 256, 0, s>>>(R, a.Rt, d, Rinv, st);
     const int nt = (d + 31) / 32;
     k_form_hinv<<<dim3(nt, nt), 256, 0, s>>>(Rinv, d, Hinv);
+    launched += 2;
   }
   return cudaGetLastError();
 }

@@ -332,9 +332,10 @@ cudaError_t launch_cluster(void (*kern)(P...), unsigned grid, unsigned threads, 
 
 // Two columns per CTA while that fills the GPU (each CTA reads all of V), one below, and the rows of a
 // column over a cluster when few columns are left.
-cudaError_t launch_trail(const TrailArgs &a, cudaStream_t s) {
+cudaError_t launch_trail(const TrailArgs &a, cudaStream_t s, int &launched) {
   const int n = a.c1 - a.c0;
   if (n <= 0) return cudaSuccess;
+  ++launched;
   if (n <= 38) return launch_cluster(k_qr_trail<1, 4>, 4u * n, kThreads, 4, kTrailSmem, s, a);
   if (n <= 76) return launch_cluster(k_qr_trail<1, 2>, 2u * n, kThreads, 2, kTrailSmem, s, a);
   if (n <= 152) k_qr_trail<1, 1><<<n, kThreads, kTrailSmem, s>>>(a);
@@ -354,7 +355,7 @@ size_t qr_panels_ws_bytes(int64_t r, int d) {
 }
 
 cudaError_t launch_qr_panels(const double *A, int64_t r, int d, int64_t lda, double *R, double *Rt, void *ws, DevState *st,
-                             cudaStream_t s) {
+                             cudaStream_t s, int &launched) {
   const int64_t ldr = ld_rows(r);
   char *p = static_cast<char *>(ws);
   double *At = reinterpret_cast<double *>(p);
@@ -402,21 +403,23 @@ cudaError_t launch_qr_panels(const double *A, int64_t r, int d, int64_t lda, dou
     e = launch_cluster(per <= kThreads ? k_qr_panel<1> : (per <= 2 * kThreads ? k_qr_panel<2> : k_qr_panel<4>), kCluster,
                        threads, kCluster, kPanelSmem, sc, pa);
     if (e != cudaSuccess) return e;
+    ++launched;
     TrailArgs ta{At, ldr, j0, r - j0, c0, c1, V[blk], T[blk]};
     // the block before has reached the next panel's columns
     if (ahead && j0 > 0 && (e = cudaStreamWaitEvent(sc, e_rest, 0))) return e;
-    if ((e = launch_trail(ta, sc)) != cudaSuccess) return e;
+    if ((e = launch_trail(ta, sc, launched)) != cudaSuccess) return e;
     ta.c0 = c1;
     ta.c1 = d;
     // the columns behind wait for that too: the next panel, of the higher priority, is placed first
     if (ahead && ((e = cudaEventRecord(e_chain, sc)) || (e = cudaStreamWaitEvent(s, e_chain, 0)))) return e;
-    if ((e = launch_trail(ta, s)) != cudaSuccess) return e;
+    if ((e = launch_trail(ta, s, launched)) != cudaSuccess) return e;
     if (ahead && (e = cudaEventRecord(e_rest, s))) return e;
   }
   if (ahead) {
     if ((e = cudaEventRecord(e_chain, sc)) || (e = cudaStreamWaitEvent(s, e_chain, 0))) return e;
   }
   k_qr_extract<<<(d * d + 255) / 256, 256, 0, s>>>(At, ldr, d, R, Rt);
+  launched += 2;  // with the transpose
   return cudaGetLastError();
 }
 

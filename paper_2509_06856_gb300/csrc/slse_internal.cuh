@@ -184,6 +184,7 @@ CsPlan cs_plan(int64_t N, int d, int prec, int64_t m_min, int64_t m_max, int64_t
 cudaError_t launch_countsketch(const CsPlan &pl, int xdtype, const void *X, int64_t ldx, const void *Y, uint64_t seed,
                                void *const *lvX, void *const *lvY, int64_t ldo, void *hatX, void *hatY, int64_t ldh,
                                void *ws, cudaStream_t s);
+int cs_kernels(const CsPlan &pl);  // kernels of that call: sort; starts, top levels, folds; Hessian sketch
 
 // fp8.cu: the FP8 form of the sketch (E4M3 values, one power-of-two scale per 32-column
 // block of a row, byte = exponent + 127; Y values in BF16).
@@ -344,15 +345,16 @@ cudaError_t launch_copy_beta(const double *beta_ring, DevState *st, int d, doubl
 // not modified); r within qr_panels_ok.  An exactly zero column raises ST_NUMERIC.
 bool qr_panels_ok(int64_t r);
 size_t qr_panels_ws_bytes(int64_t r, int d);
+// Adds the kernels it launches to `launched`.
 cudaError_t launch_qr_panels(const double *A, int64_t r, int d, int64_t lda, double *R, double *Rt, void *ws, DevState *st,
-                             cudaStream_t s);
+                             cudaStream_t s, int &launched);
 
 // linalg.cu
 size_t qr_ws_bytes(int64_t r, int d, int nsm);
 cudaError_t launch_gather_hessian_rows(int prec, const void *U, int64_t ldu, int64_t row0, int64_t r,
                                        int d, double scale, double *A, cudaStream_t s);
 cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, double *Hinv, void *ws, void *panels,
-                      DevState *st, cudaStream_t s);
+                      DevState *st, cudaStream_t s, int &launched);
 // Mixed path: H-hat^{-1} = G^{-1} for G = scale2 * U[row0:row0+r]^T U[row0:row0+r] (U in BF16,
 // G accumulated exactly), by the blocked sweep operator in FP64.  A non-positive pivot
 // raises ST_NUMERIC (the caller then takes the Householder QR).
