@@ -1004,7 +1004,7 @@ __global__ void __launch_bounds__(256) k_update(const UpdArgs A, DevState *st) {
     const int k2 = t - a.hist_base;
     if (k2 >= 0 && k2 < (int)sizeof(st->mode_hist)) st->mode_hist[k2] = exact ? 0 : 1;
     if (exact) st->ns_pass += st->t_red - st->t_mark;
-    else st->ns_corr += st->t_upd - st->t_mark;
+    else st->ns_corr += st->t_upd - st->t_red;  // not the wait for the Gram matrix before the first one
     st->t_mark = device_ns();
     if (corr && exact) {
       // a cycle (exact pass + k correction steps, 1 + k c passes' worth of time for a correction
