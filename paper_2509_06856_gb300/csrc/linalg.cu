@@ -465,7 +465,7 @@ cudaError_t launch_qr(double *A, int64_t r, int d, int64_t lda, double *R, doubl
   // by panels up to 16384 rows (their rows stay in a cluster's registers); the column-by-column form
   // above that, and when a test limits the polls of its grid barrier (the panels have no such wait)
   if (panels && qr_panels_ok(r) && debug_spin_limit() == 0) {
-    if ((e = launch_qr_panels(A, r, d, lda, R, a.Rt, panels, st, s, launched)) != cudaSuccess) return e;
+    if ((e = launch_qr_panels(A, r, d, lda, R, a.Rt, panels, st, nsm, s, launched)) != cudaSuccess) return e;
   } else {
     const int64_t nr_max = (r + G - 1) / G;
     const size_t smem = (size_t)nr_max * d * sizeof(double);

@@ -331,14 +331,15 @@ cudaError_t launch_cluster(void (*kern)(P...), unsigned grid, unsigned threads, 
 }
 
 // Two columns per CTA while that fills the GPU (each CTA reads all of V), one below, and the rows of a
-// column over a cluster when few columns are left.
-cudaError_t launch_trail(const TrailArgs &a, cudaStream_t s, int &launched) {
+// column over a cluster when few columns are left: as many CTAs as there are SMs at most, until one column
+// each does not fit.
+cudaError_t launch_trail(const TrailArgs &a, int nsm, cudaStream_t s, int &launched) {
   const int n = a.c1 - a.c0;
   if (n <= 0) return cudaSuccess;
   ++launched;
-  if (n <= 38) return launch_cluster(k_qr_trail<1, 4>, 4u * n, kThreads, 4, kTrailSmem, s, a);
-  if (n <= 76) return launch_cluster(k_qr_trail<1, 2>, 2u * n, kThreads, 2, kTrailSmem, s, a);
-  if (n <= 152) k_qr_trail<1, 1><<<n, kThreads, kTrailSmem, s>>>(a);
+  if (n <= nsm / 4) return launch_cluster(k_qr_trail<1, 4>, 4u * n, kThreads, 4, kTrailSmem, s, a);
+  if (n <= nsm / 2) return launch_cluster(k_qr_trail<1, 2>, 2u * n, kThreads, 2, kTrailSmem, s, a);
+  if (n <= nsm) k_qr_trail<1, 1><<<n, kThreads, kTrailSmem, s>>>(a);
   else k_qr_trail<2, 1><<<(n + 1) / 2, kThreads, kTrailSmem, s>>>(a);
   return cudaGetLastError();
 }
@@ -355,7 +356,7 @@ size_t qr_panels_ws_bytes(int64_t r, int d) {
 }
 
 cudaError_t launch_qr_panels(const double *A, int64_t r, int d, int64_t lda, double *R, double *Rt, void *ws, DevState *st,
-                             cudaStream_t s, int &launched) {
+                             int nsm, cudaStream_t s, int &launched) {
   const int64_t ldr = ld_rows(r);
   char *p = static_cast<char *>(ws);
   double *At = reinterpret_cast<double *>(p);
@@ -407,12 +408,12 @@ cudaError_t launch_qr_panels(const double *A, int64_t r, int d, int64_t lda, dou
     TrailArgs ta{At, ldr, j0, r - j0, c0, c1, V[blk], T[blk]};
     // the block before has reached the next panel's columns
     if (ahead && j0 > 0 && (e = cudaStreamWaitEvent(sc, e_rest, 0))) return e;
-    if ((e = launch_trail(ta, sc, launched)) != cudaSuccess) return e;
+    if ((e = launch_trail(ta, nsm, sc, launched)) != cudaSuccess) return e;
     ta.c0 = c1;
     ta.c1 = d;
     // the columns behind wait for that too: the next panel, of the higher priority, is placed first
     if (ahead && ((e = cudaEventRecord(e_chain, sc)) || (e = cudaStreamWaitEvent(s, e_chain, 0)))) return e;
-    if ((e = launch_trail(ta, s, launched)) != cudaSuccess) return e;
+    if ((e = launch_trail(ta, nsm, s, launched)) != cudaSuccess) return e;
     if (ahead && (e = cudaEventRecord(e_rest, s))) return e;
   }
   if (ahead) {

@@ -347,7 +347,7 @@ bool qr_panels_ok(int64_t r);
 size_t qr_panels_ws_bytes(int64_t r, int d);
 // Adds the kernels it launches to `launched`.
 cudaError_t launch_qr_panels(const double *A, int64_t r, int d, int64_t lda, double *R, double *Rt, void *ws, DevState *st,
-                             cudaStream_t s, int &launched);
+                             int nsm, cudaStream_t s, int &launched);
 
 // linalg.cu
 size_t qr_ws_bytes(int64_t r, int d, int nsm);
