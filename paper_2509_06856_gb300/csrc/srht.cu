@@ -624,7 +624,13 @@ cudaError_t launch_pass_t(const GroupArgs &a, int L, int64_t ngroups, cudaStream
   cudaError_t e;
   // FP32 arithmetic, groups of 2^10 and 2^11 rows with 16-byte aligned rows: the tensor-core form
   // (bench shape: passes 3.45 + 3.22 ms in the cluster form, 3.00 + 1.49 ms there; 2^12 rows would leave
-  // 16 columns of tensor memory, 32-byte row segments)
+  // 16 columns of tensor memory, 32-byte row segments).  Pass 1 over groups of 2^10 rows takes 64 columns at
+  // a time, the cluster form 32: the cluster form keeps the widths whose last 64 are less than half full, and
+  // with 512 groups (N' = 2^19) those below four such slabs, where the CTAs run three to eleven tiles each.
+  // Whole sketch, us, tensor cores against cluster form in pass 1: N' = 2^20 x 32 306, 258; x 64 306, 302; x 96
+  // 433, 391; x 112 440, 459; x 224 677, 659; x 256 675, 704; N' = 2^19 x 64 226, 207; x 192 389, 379; x 256
+  // 460, 462; x 512 768, 793.  Groups of 2^11 rows (32 columns): 2^21 x 1 468, 466; x 8 469, 476; 2^22 x 24 760,
+  // 805.  Pass 2: 2^20 x 8 310, 302; x 32 306, 301 (no second form for that); x 40 313, 349; 2^22 x 8 739, 827.
   bool tc = false;
   if constexpr (std::is_same_v<Tout, __nv_bfloat16>) {
     auto ok16 = [](const void *p, int64_t ld, size_t eb) {
@@ -632,6 +638,10 @@ cudaError_t launch_pass_t(const GroupArgs &a, int L, int64_t ngroups, cudaStream
     };
     tc = (L == 10 || L == 11) && ok16(a.in, a.ldin, sizeof(Tin)) && a.ldin < (int64_t(1) << 30) &&
          (std::is_same_v<Tin, float> ? a.Psd != nullptr : a.Psd == nullptr);
+    if (std::is_same_v<Tin, float> && L == 10) {
+      const int s64 = (a.d + 63) / 64, s32 = (a.d + 31) / 32;
+      tc = tc && 2 * s64 == s32 && (ngroups >= 1024 || s64 >= 4);
+    }
     if (tc) {
       GroupArgs b = a;
       b.vec_out = ok16(a.out, a.ldout, 2) ? 1 : 0;
@@ -724,6 +734,7 @@ cudaError_t run_plan(const SrhtPlan &pl, const void *X, int64_t ldx, const void 
   a.scale = 1.0;
   a.copy_out = copy_out;
   a.vec_out = vec_ok(W, ldw, sizeof(Tout), VO) ? 1 : 0;
+  a.pad_out = ldw >= ((d + 7) & ~7) ? 1 : 0;
   cudaError_t e = copy_out ? launch_pass_t<Tin, Ts, Tout, VA, VB, VO, P1_SLAB, P1_MB, true>(a, pl.log2, n1, s)
                            : launch_pass_t<Tin, Ts, Tout, VA, VB, VO, P1_SLAB, P1_MB, false>(a, pl.log2, n1, s);
   if (e != cudaSuccess) return e;
@@ -733,6 +744,7 @@ cudaError_t run_plan(const SrhtPlan &pl, const void *X, int64_t ldx, const void 
   b.Psd = nullptr;
   b.N = 0;
   b.copy_out = nullptr;
+  b.pad_out = 0;
   b.in = W; b.ldin = ldw; b.in_y = WY;
   b.vec_in = vec_ok(W, ldw, sizeof(Tout), VA) ? 1 : 0;
   b.vec_out = vec_ok(U, ldu, sizeof(Tout), VO) ? 1 : 0;

@@ -25,6 +25,7 @@ struct GroupArgs {
   int nslab;
   int logq;
   int vec_in, vec_out;  // 1: rows allow VEC-wide vector access
+  int pad_out;          // 1: output rows have room up to a multiple of 8 columns (the intermediate W)
   uint8_t *out_scale;   // FP8 form: block exponents, ld_scale bytes per row
   int64_t ld_scale;
   __nv_bfloat16 *hat_out;  // FP8 form: output rows >= hat_row0 go here in BF16 (nullable)

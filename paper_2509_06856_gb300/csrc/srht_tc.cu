@@ -30,6 +30,8 @@
 // half the rate), all output rows read back before the first store (spills).
 // Every mbarrier wait is bounded (ST_TIMEOUT: the fit reports it, slse_sketch's output is NaN then);
 // copies in flight are awaited and tensor memory is freed on that path too.
+#include <climits>
+
 #include "srht_args.cuh"
 #include "tc_common.cuh"
 
@@ -506,6 +508,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_group_tc(const TcPassArgs A) 
       // (more does not fit the registers), and tensor memory is free for the next group
       constexpr int NU = 2 * KH, N1 = NU / 4;
       const bool fast = a.vec_out && col0 + C <= d;
+      // the last slab's units: whole while eight columns are left, and in W, whose rows are padded, up to the
+      // end (2^22 x 112, the whole sketch: 2317 us with two-byte stores there, 1602 so; 2126 in the cluster
+      // form)
+      const int nvec = !a.vec_out ? INT_MAX : (a.pad_out ? 1 : 8);
       auto read_unit = [&](int z, uint32_t *u) {
         tmem_ld_rows<2 * U>(tq + ((uint32_t)(16 * (z & 1)) << 16) + (uint32_t)((part * KH + (z >> 1)) * C), u);
       };
@@ -519,10 +525,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_group_tc(const TcPassArgs A) 
 #pragma unroll
           for (int h = 0; h < U; ++h) {
             const uint32_t *f = u + 8 * h + 2 * x;
-            if (fast) {
+            const int n = d - (col0 + (lane & 3) * 8 + 32 * h);  // columns left
+            if (fast || n >= nvec) {
               *reinterpret_cast<uint4 *>(orow + 32 * h) = make_uint4(f[0], f[1], f[4], f[5]);
             } else {
-              const int n = d - (col0 + (lane & 3) * 8 + 32 * h);  // columns left
               const uint32_t e4[4] = {f[0], f[1], f[4], f[5]};
 #pragma unroll
               for (int e = 0; e < 8; ++e)

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 def test_a_wait_that_gives_up_is_seen(N, prec):
     torch = torch_cuda()
     import paper_2509_06856_gb300 as slse
-    d, m = 20, 4096
+    d, m = 252 if N < 1 << 19 else 20, 4096  # groups of 2^10 rows: on the tensor cores from there on
     g = torch.Generator(device="cuda").manual_seed(N)
     X = torch.randn(N, d, generator=g, device="cuda")
     Y = torch.randn(N, generator=g, device="cuda")
