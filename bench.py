@@ -233,6 +233,12 @@ def e4m3_values():
     return v
 
 
+def link_rates(nbytes, ms_pass1, ms_copy):
+    """GB/s at which pass 1 read X from host memory, of a plain copy of the same X, and the share."""
+    read, copy = (nbytes / statistics.median(ms) / 1e6 for ms in (ms_pass1, ms_copy))
+    return {"pass1_host_read_gbs": read, "link_copy_gbs": copy, "pass1_frac_of_link": read / copy}
+
+
 def first_crossing(hist, ms, bh, target):
     nb = np.linalg.norm(bh)
     errs = np.linalg.norm(hist - bh[None, :], axis=1) / nb
@@ -816,18 +822,28 @@ def run_ours(args, rank, ws, local_rank):
                 ev.append((t if t is not None else r.report["ms_total"], r.report["ms_copy_in"],
                            r.report["ms_srht_pass1"]))
         del wh
+        # the link of this box beside it: copies of the same pinned X by the copy engine
+        buf, copies = torch.empty(Xh.shape, dtype=Xh.dtype, device="cuda"), []
+        for k in range(4):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            buf.copy_(Xh, non_blocking=True)
+            e1.record()
+            torch.cuda.synchronize()
+            copies.append(e0.elapsed_time(e1))
+        del buf
         if rank == 0:
             e2e = {"value": reduce_max(statistics.median(v for v, _, _ in ev), 1), "unit": "ms",
                    "h2d_bytes_per_step": int(Xh.numel() * 4 + Yh.numel() * 4), "d2h_bytes_per_step": d * 8,
                    "steps_ms": [round(v, 3) for v, _, _ in ev],
                    "ms_copy_in": statistics.mean(c for _, c, _ in ev),
                    "ms_srht_pass1_from_host": statistics.median(p1 for _, _, p1 in ev),
-                   "pass1_host_read_gbs": Xh.numel() * 4 / statistics.median(p1 for _, _, p1 in ev) / 1e6,
+                   **link_rates(Xh.numel() * 4, [p1 for _, _, p1 in ev], copies[1:]),
                    "how": "slse_fit with pinned host X, Y: Y copied on a side stream during the draws, X read from host "
                           "memory by the first SRHT pass, which also writes its device copy; "
                           "time from the call's first CUDA event to the first iterate within 1e-8; median of the "
-                          "steps; pass1_host_read_gbs is the rate at which that pass reads X over the host link "
-                          "(the link's own rate on these boxes, cudaMemcpyAsync or SM loads: 208-211 GB/s)"}
+                          "steps; pass1_host_read_gbs is the rate at which that pass reads X over the host link, "
+                          "link_copy_gbs the rate of a copy of the same pinned X by the copy engine in this run"}
 
     if rank != 0:
         return
