@@ -675,9 +675,11 @@ slse_status fit_impl(const slse_problem *pin, const Sched &s, uint64_t seed, dou
   ua.T = T;
 
   // The iteration's kernels are dependent launches (their CTAs wait in place), except beside a long Gram
-  // build: the waiting CTAs take the gaps in which its CTAs get onto the SMs.  Measured: mixed fit of
-  // 100003 x 37 1.32 -> 1.04 ms, FP64 fit of 20000 x 50 1.42 -> 1.25, CountSketch fit of 1500001 x 256
-  // 3.81 -> 3.70; 2^22 x 512 13.4 -> 14.0 ms with them beside the build (from 2 to 4.8 ms long).
+  // build, where the waiting CTAs take the gaps in which its CTAs get onto the SMs.  Measured, dependent
+  // against plain launches (us; SRHT, CountSketch): N d = 2^25 x 128 columns 1284, 1348; 1298, 1362; 2^28 x 256 2747,
+  // 2780; 2843, 2888; 2^29 x 512 4856, 4868; 5279, 5268; 2^29 x 128 5076, 5179; 2^30 x 256 6937, 7029; 7155, 7278;
+  // 2^30 x 512 7807, 7760; 8792, 8310; 2^31 x 512 13672, 13313; 15215, 14466.  The line lies where they stop
+  // gaining at every width.
   const bool dep_early = !L.dc || (double)p->N * d < 0x1p29;
   // a8 stage 1: a_i M-IHS steps on each nested sketch (prefix of the sampled rows)
   int t = 0;
