@@ -971,13 +971,10 @@ slse_status slse_sketch(const slse_problem *prob, int32_t kind, int32_t prec, ui
   int32_t *sigma = reinterpret_cast<int32_t *>(base + L.o_sigma);
   int32_t *pos = reinterpret_cast<int32_t *>(base + L.o_pos);
   CK(launch_draws(Np, seed, Psd, nullptr, sigma, nullptr, base + L.o_big, st));
-  CK(launch_pos_map(sigma, Np, 0, m, L.sp.single ? L.sp.logN : L.sp.log2, pos, st));
-  // sigma is not read any more: its first word takes the passes' status (a wait that gave up leaves NaN)
-  unsigned *status = nullptr;
-  if (!L.sp.single) {
-    status = reinterpret_cast<unsigned *>(sigma);
-    CK(cudaMemsetAsync(status, 0, sizeof(unsigned), st));
-  }
+  // sigma is not read behind the map: its first word, cleared there, takes the passes' status (a wait that
+  // gave up leaves NaN)
+  CK(launch_pos_map(sigma, Np, 0, m, L.sp.single ? L.sp.logN : L.sp.log2, pos, st, true));
+  unsigned *status = L.sp.single ? nullptr : reinterpret_cast<unsigned *>(sigma);
   if (prec == SLSE_PREC_MIXED_FP8) {
     // SX: m x ldsx E4M3 bytes followed by the m x ceil(d/32) block-exponent bytes
     uint8_t *scales = static_cast<uint8_t *>(SX) + (size_t)m * ldsx;

@@ -265,9 +265,10 @@ cudaError_t launch_draws(int64_t Np, uint64_t seed, int32_t *Psd /*N', sign-fold
                          int32_t *P /*nullable*/, int32_t *sigma, int8_t *D /*nullable*/,
                          void *ws, cudaStream_t s);
 // pos[idx(k)] = s for k = sigma[s], s in [s0, s1), -1 elsewhere; idx(k) = (k mod n2) n1 + k div n2
-// with n2 = 2^log2 (the pass-1 group size; log2 = log2 N' for single-pass plans).
-cudaError_t launch_pos_map(const int32_t *sigma, int64_t Np, int64_t s0, int64_t s1, int log2, int32_t *pos,
-                           cudaStream_t s);
+// with n2 = 2^log2 (the pass-1 group size; log2 = log2 N' for single-pass plans).  clear_first: sigma[s0]
+// is zero afterwards (a word for the caller, without a launch of its own).
+cudaError_t launch_pos_map(int32_t *sigma, int64_t Np, int64_t s0, int64_t s1, int log2, int32_t *pos, cudaStream_t s,
+                           bool clear_first = false);
 
 // srht.cu
 struct SrhtPlan {
