@@ -121,15 +121,15 @@ __device__ __forceinline__ void warp_sum_rows(double (&v)[R], int lane) {
 //    2^-7 of the row's largest).  It has the sign of its term: without it every x_i beta came out 2^-59
 //    too small, an error of the gradient along X^T X beta that grew with the rows.  Residual 1e-3 of
 //    X beta, 131072 x 10, error against a double-double sum: FP64 chain 2.6e-13, without zl bl 1.4e-12, with
-//    it 1.8e-13.  It costs 4 % at 2^20 x 256 (with all 64 bits 8 %).
+//    it 1.8e-13.  It costs 2 % at 2^20 x 256, 5 % at 2^20 x 512 (with all 64 bits 5 and 5 to 7 %).
 // The error of x_i beta is then below that of an FP64 chain (2^-53 of the partial sums at each of
 // its d steps): sqrt(d) 2^-60 of the row's largest term, and half an ulp.  A row group with a
 // denormal, an infinity or a NaN, or whose largest product is outside [2^-846, 2^954], takes the FP64
 // sums (warp-uniform).  A row without a non-zero term has the sum zero and stays here (in
 // the FP64 sums, which read X again element by element, a pass at beta = 0 took 2420 us at 2^20 x 512, FP32
 // storage 3390; now 1190 and 1180).
-// Measured (GB300), the whole call against the FP64 chain: N = 2^20, d = 256 FP64 1.10 -> 0.69 ms, d = 512
-// FP64 2.02 -> 1.25 ms, FP32 storage 2.08 -> 1.25 ms.  What bounds it now: the FP64 pipe, 0.76
+// Measured (GB300), the whole call against the FP64 chain: N = 2^20, d = 256 FP64 1.10 -> 0.67 ms, d = 512
+// FP64 2.02 -> 1.26 ms, FP32 storage 2.08 -> 1.25 ms.  What bounds it now: the FP64 pipe, 0.76
 // busy (the integer pipe 0.67).  Before zl bl (0.63 ms at 2^20 x 256): 0.69 ms without
 // the ring (rows prefetched into registers), 0.86 ms without any prefetch, 0.77 ms with three CTAs of
 // 80 registers.
@@ -230,6 +230,11 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_grad_f64(const GradArgs a) 
   const Tx *X = static_cast<const Tx *>(a.X);
   const Tx *Y = static_cast<const Tx *>(a.Y);
   constexpr int NB = BS ? 1 : VMAX * VW;
+  // A row without a non-zero term: with the largest exponent kept above the terms' every shift is large and
+  // the sums are zero by themselves (2^20 x 256 FP64 665 us, against 691 with the sum left out at the end;
+  // 2^20 x 512 FP32 1252, 1294), but with beta in shared memory the other forms schedule worse so (2^20 x
+  // 512 FP64 1350, 1254; 2^20 x 511 FP32 1534, 1408), and the sum is left out.
+  constexpr bool kClamp = !BS || (sizeof(Tx) == 4 && VW == 2);
   int rbh[NB], rbl[NB], rbe[NB];
   // shared-memory form: (bh, bl) pairs, then the exponents, in lane order
   int2 *sb = reinterpret_cast<int2 *>(&sm[0][0]);
@@ -322,6 +327,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_grad_f64(const GradArgs a) 
           fmax = max(fmax, f[v][e]);
         }
       fmax = __reduce_max_sync(0xffffffffu, fmax);
+      if constexpr (kClamp) fmax = max(fmax, kNoTerm / 2);
       long long sh = 0, s1 = 0, s2 = 0;
       int s3 = 0;
 #pragma unroll
@@ -359,12 +365,12 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_grad_f64(const GradArgs a) 
       const uint32_t q1 = __reduce_add_sync(0xffffffffu, __funnelshift_r(w0, w1, 26) & 0x3FFFFFFu);
       const uint32_t q2 = __reduce_add_sync(0xffffffffu, __funnelshift_r(w1, w2, 20) & 0x3FFFFFFu);
       const int q3 = __reduce_add_sync(0xffffffffu, (int)w2 >> 14);
-      if (lane == q) { p0 = q0; p1 = q1; p2 = q2; p3 = q3; F = fmax; }
+      if (lane == q) { p0 = q0; p1 = q1; p2 = q2; p3 = q3; F = kClamp && fmax == kNoTerm / 2 ? 1200 : fmax; }
     }
     const bool rv = lane < RPW && i0 + lane < a.nrows;
     odd = __any_sync(0xffffffffu, odd);
     double r[RPW];
-    const bool none = F < kNoTerm / 2;  // no non-zero term: a row of zeros, or beta = 0
+    const bool none = !kClamp && F < kNoTerm / 2;  // no non-zero term: a row of zeros, or beta = 0
     if (!beta_odd && !odd && !__any_sync(0xffffffffu, rv && !none && (uint32_t)(F - 1200) > 1800u)) {
       const double rl = rv ? (none ? y : y - dot_total(p0, p1, p2, p3, F)) : 0.0;
 #pragma unroll
