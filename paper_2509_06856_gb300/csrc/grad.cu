@@ -233,8 +233,9 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_grad_f64(const GradArgs a) 
   // A row without a non-zero term: with the largest exponent kept above the terms' every shift is large and
   // the sums are zero by themselves (2^20 x 256 FP64 665 us, against 691 with the sum left out at the end;
   // 2^20 x 512 FP32 1252, 1294), but with beta in shared memory the other forms schedule worse so (2^20 x
-  // 512 FP64 1350, 1254; 2^20 x 511 FP32 1534, 1408), and the sum is left out.
-  constexpr bool kClamp = !BS || (sizeof(Tx) == 4 && VW == 2);
+  // 512 FP64 1350, 1254; 2^20 x 511 FP32 1534, 1408), and the narrowest tile, whose passes are short, feels its
+  // latency (an FP64 fit of 20000 x 50 1221, 1157): there the sum is left out.
+  constexpr bool kClamp = BS ? sizeof(Tx) == 4 && VW == 2 : VMAX >= 2;
   int rbh[NB], rbl[NB], rbe[NB];
   // shared-memory form: (bh, bl) pairs, then the exponents, in lane order
   int2 *sb = reinterpret_cast<int2 *>(&sm[0][0]);
