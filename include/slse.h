@@ -296,7 +296,8 @@ int32_t slse_default_schedule_for(int64_t N, int32_t d, int32_t kind, slse_sched
  * its sizes m, a, kind and its stage2 are ignored.  X device; Y unused.  v, w_out: device d doubles.
  * report (nullable): ms_total, iters_stage2, final_rel_step, rebases, status.  Returns after w_out
  * is written (SLSE_ENOTCONV if tol > 0 was not met within T, w_out holds the last iterate).
- * Workspace: slse_solve_normal_workspace bytes, or NULL for a stream-ordered allocation. */
+ * Workspace: slse_solve_normal_workspace bytes, or NULL for a stream-ordered allocation (F32 X of 2^24
+ * elements and more with MIXED_BF16: 8 d^2 bytes less are enough). */
 slse_status slse_solve_normal(const slse_problem *prob, const double *Hinv, const double *v, double *w_out,
                               const slse_schedule *sched, slse_report *report, void *workspace, size_t ws_bytes,
                               slse_stream_t stream);

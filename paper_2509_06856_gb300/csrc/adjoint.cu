@@ -272,8 +272,8 @@ AdjLayout adj_layout(const slse_problem *p, int prec, int nsm) {
   L.o_r0 = take(prec == SLSE_PREC_MIXED_BF16 ? (size_t)p->N * 4 : 0);
   L.o_y0 = take((size_t)p->N * (p->dtype == SLSE_F64 ? 8 : 4));
   L.total = o;
-  // The query has room for a d x d matrix on top for large X on the mixed path (at most 2 MB): callers
-  // have been told that a workspace shorter than the query by that much is accepted.
+  // The query has room for a d x d matrix on top for large X on the mixed path (at most 2 MB), and a
+  // workspace shorter than the query by that much is accepted, as it was while the solve had a use for it.
   const bool room = prec == SLSE_PREC_MIXED_BF16 && p->dtype == SLSE_F32 && p->N * d >= (int64_t(1) << 24);
   L.query = L.total + (room ? al((size_t)d * d * 8) : 0);
   return L;
